@@ -2,11 +2,25 @@
 // reference engine for every GemmDesc shape the tensor-core engine handles.
 //
 // C(m, n) = sum_k A(m, k) B(n, k) with arbitrary element strides, grouped
-// along M (per-expert row ranges), along K (per-expert reduction ranges) or
-// dense, plus the router / SwiGLU epilogues, and the row gathers of GemmDesc.  Tile 64 x 128 x 16, 256
-// threads; thread (ty, tx) owns rows 4 ty .. 4 ty + 3 and columns
-// 4 tx .. 4 tx + 3 and 64 + 4 tx .. 64 + 4 tx + 3 of the tile, so a packed
-// gate column and its up column (64 apart) land in the same thread.
+// along M (per-expert row ranges), along K (per-expert or equal reduction
+// ranges) or dense, plus the router / SwiGLU epilogues, and the row gathers of
+// GemmDesc.  256 threads per BM x BN tile in a 16 x 16 arrangement; a thread
+// owns BM / 16 rows (in groups of up to 4, 64 apart) and BN / 16 columns (the
+// same), so that in a 128-column tile a packed gate column and its up column
+// (64 apart) land in the same thread.
+//
+// Both operands are staged in shared memory as [k][m] and [k][n], two buffers:
+// the next k-tile's global loads are issued before the current one is
+// multiplied and written to the other buffer after it, one barrier per k-tile.
+// The products are packed fp32 FMAs on two adjacent columns (fma.rn.f32x2, each
+// half rounded as a scalar FMA), in the order of k.
+//
+// Bound by the FMA pipe and its issue slots.  Measured on an fp32 layer of
+// T = 3001, D = 512, E = 12, K = 3, F = 768: GEMM-1 (14.2 GFLOP) 526 us on the
+// single-buffered 64 x 128 x 16 tiles used before, 358 us with scalar FMAs here,
+// 320 us with packed ones (44 TFLOP/s; the FMA pipe 66 % busy, 92 % of the tile
+// rows real).  A k-tile of 8 (363 us) or 32 (336 us, spills), and one block per
+// SM with more registers (365 us), are slower.
 #include "common.cuh"
 #include "launch.h"
 
@@ -14,161 +28,376 @@ namespace moe {
 
 namespace {
 
-constexpr int BM = 64, BN = 128, BK = 16;
-
 template <typename T>
-__device__ __forceinline__ float ldf(const void* p, int64_t i) {
-  return to_f32<T>(static_cast<const T*>(p)[i]);
+__device__ __forceinline__ float ldf(const T* p) {
+  return to_f32<T>(__ldg(p));
+}
+// Four consecutive elements (16-byte aligned fp32, 8-byte aligned bf16).
+__device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 ld4(const bf16* p) {
+  const uint2 w = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                     __uint_as_float(w.y & 0xffff0000u));
+}
+__device__ __forceinline__ void st4(float* p, const float* v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void st4(bf16* p, const float* v) {
+  uint2 w;
+  w.x = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[0])) |
+        ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[1])) << 16);
+  w.y = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[2])) |
+        ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[3])) << 16);
+  *reinterpret_cast<uint2*>(p) = w;
 }
 
 __device__ __forceinline__ float silu_f(float v) { return v / (1.0f + __expf(-v)); }
 
-template <typename TA, typename TB, typename TC>
-__global__ void __launch_bounds__(256) simt_gemm_kernel(GemmDesc d) {
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Bs[BK][BN + 4];
+// One operand tile, ROWS (m or n) x BK, staged as s[k * ROWS + (row ^ swz(k))].
+// swz spreads the scalar stores of a k-contiguous operand (4 k values of one
+// row per thread, 32 / (BK / 4) rows and all BK / 4 k-chunks per warp) over
+// all 32 banks; it is a multiple of 4, so 4-row vectors stay whole.
+template <int BK>
+__device__ __forceinline__ constexpr int swz(int k) {
+  return ((k >> 2) % (BK / 4)) * (32 / (BK / 4));
+}
+
+template <typename T, int ROWS, int BK>
+struct Loader {
+  static constexpr int NV = ROWS * BK / 4 / 256;  // 4-element vectors per thread
+  static_assert(NV >= 1 && ROWS * BK == NV * 1024, "whole vectors per thread");
+  const T* p;            // the operand, advanced to this tile's group
+  int64_t s_r, s_k;      // element strides of the row and of k
+  int64_t r0, r_end;     // the tile's first row and the end of its rows
+  const int32_t* gat_r;  // row indirection of the rows / of k (or NULL)
+  const int32_t* gat_k;
+  bool kfast;            // s_k == 1: vectors along k; else along the rows
+  bool vec;              // vectors may be read whole (alignment)
+  // the fast path: this thread's vectors of the next whole k-tile, each either
+  // inside the operand or (bit clear) past its rows
+  const T* ptr[NV];
+  uint32_t in;
+  bool fast;
+
+  __device__ __forceinline__ int row_of(int j) const {
+    const int i = (int)threadIdx.x + j * 256;
+    return kfast ? i / (BK / 4) : (i % (ROWS / 4)) * 4;
+  }
+  __device__ __forceinline__ int k_of(int j) const {
+    const int i = (int)threadIdx.x + j * 256;
+    return kfast ? (i % (BK / 4)) * 4 : i / (ROWS / 4);
+  }
+  __device__ __forceinline__ void init(const T* base, int64_t sr, int64_t sk, int64_t row0, int64_t row_end,
+                                       int64_t kbeg, const int32_t* gr, const int32_t* gk) {
+    p = base;
+    s_r = sr;
+    s_k = sk;
+    r0 = row0;
+    r_end = row_end;
+    gat_r = gr;
+    gat_k = gk;
+    kfast = sk == 1;
+    // whole vectors start at a multiple of 4 along the unit-stride dimension
+    const int64_t pitch = kfast ? sr : sk, origin = kfast ? kbeg : row0;
+    vec = (kfast || sr == 1) && pitch % 4 == 0 && origin % 4 == 0 &&
+          (reinterpret_cast<uintptr_t>(base) & (4 * sizeof(T) - 1)) == 0;
+    fast = vec && !gr && !gk;
+    in = 0;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const int64_t r = row0 + row_of(j);
+      ptr[j] = base + r * sr + (kbeg + k_of(j)) * sk;
+      if (r < row_end) in |= 1u << j;
+      if (!kfast && r < row_end && r + 4 > row_end) fast = false;  // a vector across the last row
+    }
+  }
+  // The k-tile [k0, k0 + BK) cut at kend; called for consecutive k-tiles.
+  __device__ __forceinline__ void load(int64_t k0, int64_t kend, float (&v)[NV][4]) {
+    if (fast && k0 + BK <= kend) {
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (in >> j & 1u) q = ld4(ptr[j]);
+        ptr[j] += (int64_t)BK * s_k;
+        v[j][0] = q.x; v[j][1] = q.y; v[j][2] = q.z; v[j][3] = q.w;
+      }
+      return;
+    }
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const int64_t r = r0 + row_of(j), k = k0 + k_of(j);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[j][u] = 0.f;
+      if (r >= r_end || k >= kend) continue;
+      if (kfast) {
+        const T* row = p + (gat_r ? (int64_t)__ldg(gat_r + r) : r) * s_r;
+        if (vec && !gat_k && k + 4 <= kend) {
+          const float4 q = ld4(row + k);
+          v[j][0] = q.x; v[j][1] = q.y; v[j][2] = q.z; v[j][3] = q.w;
+        } else {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (k + u < kend) v[j][u] = ldf<T>(row + (gat_k ? (int64_t)__ldg(gat_k + k + u) : k + u));
+        }
+      } else {
+        const T* col = p + (gat_k ? (int64_t)__ldg(gat_k + k) : k) * s_k;
+        if (vec && !gat_r && r + 4 <= r_end) {
+          const float4 q = ld4(col + r);
+          v[j][0] = q.x; v[j][1] = q.y; v[j][2] = q.z; v[j][3] = q.w;
+        } else {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (r + u < r_end) v[j][u] = ldf<T>(col + (gat_r ? (int64_t)__ldg(gat_r + r + u) : r + u) * s_r);
+        }
+      }
+    }
+  }
+  __device__ __forceinline__ void store(float* s, const float (&v)[NV][4]) const {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const int r = row_of(j), k = k_of(j);
+      const int rs = r ^ swz<BK>(k);  // k .. k + 3 of a k-contiguous vector share it
+      if (kfast) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s[(k + u) * ROWS + rs] = v[j][u];
+      } else {
+        *reinterpret_cast<float4*>(s + k * ROWS + rs) = make_float4(v[j][0], v[j][1], v[j][2], v[j][3]);
+      }
+    }
+  }
+};
+
+// A thread's N = TILE / 16 positions of one tile dimension: t in 0 .. 15.
+template <int N>
+__device__ __forceinline__ int pos(int t, int i) {
+  return N >= 4 ? (i >> 2) * 64 + t * 4 + (i & 3) : t * N + i;
+}
+template <int N>
+__device__ __forceinline__ void frag(const float* row, int t, int sw, float (&f)[N]) {
+  if (N >= 4) {
+#pragma unroll
+    for (int g = 0; g < N / 4; ++g) {
+      const float4 q = *reinterpret_cast<const float4*>(row + ((g * 64 + t * 4) ^ sw));
+      f[4 * g] = q.x; f[4 * g + 1] = q.y; f[4 * g + 2] = q.z; f[4 * g + 3] = q.w;
+    }
+  } else {
+    const float2 q = *reinterpret_cast<const float2*>(row + ((t * 2) ^ sw));
+    f[0] = q.x; f[1] = q.y;
+  }
+}
+
+template <typename TA, typename TB, typename TC, int BM, int BN, int BK>
+__global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) simt_gemm_kernel(GemmDesc d) {
+  constexpr int TM = BM / 16, TN = BN / 16;
+  extern __shared__ __align__(16) float smem[];  // two A tiles, then two B tiles
+  auto As = [&](int b) { return smem + b * BK * BM; };
+  auto Bs = [&](int b) { return smem + 2 * BK * BM + b * BK * BN; };
+  __shared__ int s_wsum[8];
+  __shared__ int s_g;
+  __shared__ int s_row0, s_rend;
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
-  const int64_t n0 = (int64_t)blockIdx.x * BN;
+  const int tiles_n = (int)((d.N + BN - 1) / BN);
+  const int mt = (int)(blockIdx.x / (unsigned)tiles_n);  // a row tile's column tiles are consecutive blocks
+  const int64_t n0 = (int64_t)(blockIdx.x % (unsigned)tiles_n) * BN;
 
   int g = 0;
-  int64_t row0 = 0, row_end = d.M, kbeg = 0, kend = d.K;
+  int64_t row0 = (int64_t)mt * BM, row_end = d.M, kbeg = 0, kend = d.K;
   if (d.group == Group::M) {
-    const int64_t mt = blockIdx.y;
-    int64_t acc = 0;
-    g = -1;
-    for (int e = 0; e < d.num_groups; ++e) {
-      const int64_t lo = d.offsets[e], hi = d.offsets[e + 1];
-      const int64_t nt = (hi - lo + BM - 1) / BM;
-      if (mt < acc + nt) {
-        g = e;
-        row0 = lo + (mt - acc) * BM;
-        row_end = hi;
-        break;
-      }
-      acc += nt;
+    // the expert whose tiles include this one: thread e counts expert e's
+    // tiles, an exclusive scan over the (at most 256) experts places them
+    const int lane = tid & 31, warp = tid >> 5;
+    int lo = 0, hi = 0;
+    if (tid < d.num_groups) {
+      lo = __ldg(d.offsets + tid);
+      hi = __ldg(d.offsets + tid + 1);
     }
+    const int nt = (hi - lo + BM - 1) / BM;
+    int inc = nt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) s_wsum[warp] = inc;
+    if (tid == 0) s_g = -1;
+    __syncthreads();
+    int base = 0;
+    for (int w = 0; w < warp; ++w) base += s_wsum[w];
+    const int first = base + inc - nt;
+    if (mt >= first && mt < first + nt) {
+      s_g = tid;
+      s_row0 = lo + (mt - first) * BM;
+      s_rend = hi;
+    }
+    __syncthreads();
+    g = s_g;
     if (g < 0) return;
+    row0 = s_row0;
+    row_end = s_rend;
   } else if (d.group == Group::K) {
-    g = blockIdx.z;
-    row0 = (int64_t)blockIdx.y * BM;
-    kbeg = d.offsets[g];
-    kend = d.offsets[g + 1];
-  } else {
-    row0 = (int64_t)blockIdx.y * BM;
+    g = blockIdx.y;
+    if (d.offsets) {
+      kbeg = d.offsets[g];
+      kend = d.offsets[g + 1];
+    } else {
+      kbeg = d.split_rows * g / d.num_groups;
+      kend = d.split_rows * (g + 1) / d.num_groups;
+    }
   }
   if (row0 >= row_end || n0 >= d.N) return;
 
-  const void* Bp = static_cast<const char*>(d.B) + (int64_t)g * d.sb_g * sizeof(TB);
-  const bool a_kfast = d.sa_k == 1;
-  const bool b_kfast = d.sb_k == 1;
+  Loader<TA, BM, BK> la;
+  Loader<TB, BN, BK> lb;
+  la.init(static_cast<const TA*>(d.A), d.sa_m, d.sa_k, row0, row_end, kbeg,
+          d.group == Group::M ? d.gather : nullptr, nullptr);
+  lb.init(static_cast<const TB*>(d.B) + (int64_t)g * d.sb_g, d.sb_n, d.sb_k, n0, d.N, kbeg,
+          nullptr, d.group == Group::K ? d.gather : nullptr);
 
-  float acc[4][8];
+  unsigned long long acc2[TM][TN / 2];  // two adjacent columns per 64-bit pair
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < TN / 2; ++j) acc2[i][j] = 0ull;
 
+  float va[Loader<TA, BM, BK>::NV][4], vb[Loader<TB, BN, BK>::NV][4];
+  la.load(kbeg, kend, va);
+  lb.load(kbeg, kend, vb);
+  la.store(As(0), va);
+  lb.store(Bs(0), vb);
+  __syncthreads();
+  int buf = 0;
   for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
-    for (int i = tid; i < BM * BK; i += 256) {
-      int m, k;
-      if (a_kfast) { k = i % BK; m = i / BK; } else { m = i % BM; k = i / BM; }
-      const int64_t gm = row0 + m, gk = k0 + k;
-      float v = 0.f;
-      if (gm < row_end && gk < kend) {
-        const int64_t sm = (d.gather && d.group == Group::M) ? (int64_t)d.gather[gm] : gm;
-        v = ldf<TA>(d.A, sm * d.sa_m + gk * d.sa_k);
-      }
-      As[k][m] = v;
+    const bool more = k0 + BK < kend;
+    if (more) {
+      la.load(k0 + BK, kend, va);
+      lb.load(k0 + BK, kend, vb);
     }
-    for (int i = tid; i < BN * BK; i += 256) {
-      int n, k;
-      if (b_kfast) { k = i % BK; n = i / BK; } else { n = i % BN; k = i / BN; }
-      const int64_t gn = n0 + n, gk = k0 + k;
-      float v = 0.f;
-      if (gn < d.N && gk < kend) {
-        const int64_t sk = (d.gather && d.group == Group::K) ? (int64_t)d.gather[gk] : gk;
-        v = ldf<TB>(Bp, gn * d.sb_n + sk * d.sb_k);
-      }
-      Bs[k][n] = v;
-    }
-    __syncthreads();
+    const float* as = As(buf);
+    const float* bs = Bs(buf);
 #pragma unroll
     for (int k = 0; k < BK; ++k) {
-      float a[4], b[8];
+      float a[TM], b[TN];
+      frag<TM>(as + k * BM, ty, swz<BK>(k), a);
+      frag<TN>(bs + k * BN, tx, swz<BK>(k), b);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[k][ty * 4 + i];
+      for (int i = 0; i < TM; ++i) {
+        unsigned long long aa;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(a[i]));
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        b[j] = Bs[k][tx * 4 + j];
-        b[4 + j] = Bs[k][64 + tx * 4 + j];
+        for (int j = 0; j < TN / 2; ++j) {
+          unsigned long long bb;
+          asm("mov.b64 %0, {%1, %2};" : "=l"(bb) : "f"(b[2 * j]), "f"(b[2 * j + 1]));
+          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc2[i][j]) : "l"(aa), "l"(bb));
+        }
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
-    __syncthreads();
+    if (more) {
+      la.store(As(buf ^ 1), va);
+      lb.store(Bs(buf ^ 1), vb);
+      __syncthreads();
+      buf ^= 1;
+    }
   }
 
-  TC* C = static_cast<TC*>(d.C) + (d.group == Group::K ? (int64_t)g * d.sc_g : 0);
+  float acc[TM][TN];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t gm = row0 + ty * 4 + i;
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN / 2; ++j)
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[i][2 * j]), "=f"(acc[i][2 * j + 1]) : "l"(acc2[i][j]));
+  TC* C = static_cast<TC*>(d.C) + (d.group == Group::K ? (int64_t)g * d.sc_g : 0);
+  const bool vec_c = d.ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(C) & (4 * sizeof(TC) - 1)) == 0;
+  constexpr int CG = TN >= 4 ? 4 : TN;  // consecutive columns of a thread
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const int64_t gm = row0 + pos<TM>(ty, i);
     if (gm >= row_end) continue;
     TC* crow = C + gm * d.ldc;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int64_t col = (j < 4) ? (tx * 4 + j) : (64 + tx * 4 + (j - 4));
-      const int64_t gn = n0 + col;
+    for (int j0 = 0; j0 < TN; j0 += CG) {
+      const int64_t gn = n0 + pos<TN>(tx, j0);
       if (gn >= d.N) continue;
-      float v = acc[i][j];
-      switch (d.epi) {
-        case Epi::Store:
-          crow[gn] = from_f32<TC>(v);
-          break;
-        case Epi::StoreBias:
-          crow[gn] = from_f32<TC>(v + (d.bias ? d.bias[gn] : 0.f));
-          break;
-        case Epi::Accum:
-          crow[gn] = from_f32<TC>(to_f32<TC>(crow[gn]) + v);
-          break;
-        case Epi::SwigluFwd: {
-          crow[gn] = from_f32<TC>(v);
-          if (j < 4) {
-            // gate at tile column c < 64, up at c + 64 (same thread, index j + 4)
-            const float gt = v, up = acc[i][j + 4];
-            const int64_t f = n0 / 2 + col;
-            static_cast<TC*>(d.aux)[gm * (d.N / 2) + f] = from_f32<TC>(silu_f(gt) * up);
-          }
-          break;
+      const bool whole = CG == 4 && vec_c && gn + 4 <= d.N;
+      float v[CG];
+#pragma unroll
+      for (int u = 0; u < CG; ++u) {
+        v[u] = acc[i][j0 + u];
+        if (d.epi == Epi::StoreBias && d.bias && gn + u < d.N) v[u] += d.bias[gn + u];
+        if (d.epi == Epi::Accum && gn + u < d.N) v[u] = to_f32<TC>(crow[gn + u]) + v[u];
+      }
+      if (whole) {
+        if constexpr (CG == 4) st4(crow + gn, v);
+      } else {
+#pragma unroll
+        for (int u = 0; u < CG; ++u)
+          if (gn + u < d.N) crow[gn + u] = from_f32<TC>(v[u]);
+      }
+      if (d.epi == Epi::ReluSqFwd) {
+#pragma unroll
+        for (int u = 0; u < CG; ++u) {
+          const float r = fmaxf(v[u], 0.f);
+          if (gn + u < d.N) static_cast<TC*>(d.aux)[gm * d.ldc + gn + u] = from_f32<TC>(r * r);
         }
-        case Epi::ReluSqFwd: {
-          crow[gn] = from_f32<TC>(v);
-          const float r = fmaxf(v, 0.f);
-          static_cast<TC*>(d.aux)[gm * d.ldc + gn] = from_f32<TC>(r * r);
-          break;
+      }
+      if constexpr (TN == 8) {
+        // gate at tile columns c < 64, up at c + 64 (the same thread, index + 4)
+        if (d.epi == Epi::SwigluFwd && j0 == 0) {
+          TC* arow = static_cast<TC*>(d.aux) + gm * (d.N / 2) + n0 / 2 + tx * 4;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = silu_f(v[u]) * acc[i][4 + u];
+          st4(arow, v);  // N is a multiple of 128: aligned
         }
       }
     }
   }
 }
 
+template <typename TA, typename TB, typename TC, int BM, int BN, int BK>
+cudaError_t run_tile(const Ctx& c, const GemmDesc& d) {
+  const int64_t tiles_n = (d.N + BN - 1) / BN;
+  const int64_t tiles_m =
+      d.group == Group::M ? (d.max_rows + BM - 1) / BM + d.num_groups : (d.M + BM - 1) / BM;
+  const int64_t tiles = tiles_m * tiles_n;
+  const int groups = d.group == Group::K ? d.num_groups : 1;
+  if (tiles <= 0 || groups <= 0) return cudaSuccess;
+  if (tiles > 0x7fffffff) return cudaErrorInvalidConfiguration;
+  const dim3 grid((unsigned)tiles, (unsigned)groups, 1);
+  constexpr int kSmem = 2 * (BM + BN) * BK * 4;
+  static_assert(kSmem <= 48 * 1024, "fits without opting in to more shared memory");
+  simt_gemm_kernel<TA, TB, TC, BM, BN, BK><<<grid, 256, kSmem, c.stream>>>(d);
+  return cudaGetLastError();
+}
+
+// Tiles of a BM x BN tiling that hold rows (an upper estimate for Group::M,
+// whose experts' row counts only the device knows).
+int64_t tiles_of(const GemmDesc& d, int bm, int bn) {
+  const int64_t nt = (d.N + bn - 1) / bn;
+  if (d.group == Group::M) {
+    const int64_t groups = d.max_rows < d.num_groups ? d.max_rows : d.num_groups;
+    return nt * (d.max_rows / bm + (groups + 1) / 2);
+  }
+  return nt * ((d.M + bm - 1) / bm) * (d.group == Group::K ? d.num_groups : 1);
+}
+
 template <typename TA, typename TB, typename TC>
 cudaError_t run(const Ctx& c, const GemmDesc& d) {
-  dim3 block(256);
-  dim3 grid((unsigned)((d.N + BN - 1) / BN), 1, 1);
-  if (d.group == Group::M) {
-    grid.y = (unsigned)((d.max_rows + BM - 1) / BM + d.num_groups);
-  } else if (d.group == Group::K) {
-    grid.y = (unsigned)((d.M + BM - 1) / BM);
-    grid.z = (unsigned)d.num_groups;
+  const bool swiglu = d.epi == Epi::SwigluFwd;  // needs gate and up columns in one 128-column tile
+  if constexpr (sizeof(TA) == 4 && sizeof(TB) == 4) {
+    // the largest tile that still gives every SM work: at T = 256, D = 128, E = 8,
+    // K = 2, F = 256 the small tiles take GEMM-1's dgrad from 102 to 17 us
+    if (d.N > 64) {
+      if (tiles_of(d, 128, 128) >= c.num_sms) return run_tile<TA, TB, TC, 128, 128, 16>(c, d);
+      if (tiles_of(d, 64, 128) >= c.num_sms) return run_tile<TA, TB, TC, 64, 128, 16>(c, d);
+      if (swiglu) return run_tile<TA, TB, TC, 32, 128, 32>(c, d);
+    }
+    if (tiles_of(d, 64, 64) >= c.num_sms && d.N > 32) return run_tile<TA, TB, TC, 64, 64, 32>(c, d);
+    return run_tile<TA, TB, TC, 32, 32, 32>(c, d);
   } else {
-    grid.y = (unsigned)((d.M + BM - 1) / BM);
+    if (swiglu || (d.N > 64 && tiles_of(d, 64, 128) >= c.num_sms))
+      return run_tile<TA, TB, TC, 64, 128, 16>(c, d);
+    return run_tile<TA, TB, TC, 32, 32, 32>(c, d);
   }
-  if (grid.x == 0 || grid.y == 0 || grid.z == 0) return cudaSuccess;
-  simt_gemm_kernel<TA, TB, TC><<<grid, block, 0, c.stream>>>(d);
-  return cudaGetLastError();
 }
 
 }  // namespace
