@@ -195,6 +195,16 @@ int router_splits(const Dims& d, int num_sms) {
   if (s > d.T / 256) s = d.T / 256;
   return s < 1 ? 1 : (int)s;
 }
+// The same for the CUDA-core engine (fp32 inputs, or a number of experts that
+// the tensor-core engine does not take), which covers a thin output with 32 x 32
+// tiles: the three blocks per SM that fit, each reducing at least 256 tokens.
+int router_splits_simt(const Dims& d, int num_sms) {
+  const int64_t tiles = (int64_t)((d.E + 31) / 32) * ((d.Din + 31) / 32);
+  int64_t s = 3 * num_sms / tiles;
+  if (s > kRouterSplits) s = kRouterSplits;
+  if (s > d.T / 256) s = d.T / 256;
+  return s < 1 ? 1 : (int)s;
+}
 // Sigmoid router forward: per-token score sums and the balance statistics'
 // per-chunk partial sums.
 size_t ws_route_sigmoid(const Dims& d) { return align_up(route_sigmoid_fwd_ws_bytes(d.T, d.S, d.GBS, d.E)); }
@@ -876,6 +886,22 @@ static int router_grad_gemms(const Ctx& c, const Dims& d, const void* x, const v
       TRY_CUDA(launch_sum_splits(c, static_cast<const float*>(bs.C), splits, (int64_t)d.E * d.Din, dw_router));
       return MOE_OK;
     }
+  }
+  const int simt_splits = gemm_tc_supports(b) ? 1 : router_splits_simt(d, c.num_sms);
+  if (simt_splits > 1) {
+    // the same split for the CUDA-core engine: without it the few tiles of an
+    // E x Din output each walk all T tokens (fp32 T = 3001, E = 12, Din = 512:
+    // 627 us; bf16 T = 2045, E = 60, Din = 2048: 451 us; now 17 and 44 us)
+    GemmDesc bs = b;
+    bs.group = Group::K;
+    bs.num_groups = simt_splits;
+    bs.offsets = nullptr;
+    bs.split_rows = d.T;
+    bs.C = scratch;
+    bs.sc_g = (int64_t)d.E * d.Din;
+    TRY_CUDA(launch_gemm_simt(c, bs, "router_wgrad_simt"));
+    TRY_CUDA(launch_sum_splits(c, static_cast<const float*>(bs.C), simt_splits, (int64_t)d.E * d.Din, dw_router));
+    return MOE_OK;
   }
   TRY_CUDA(gemm(c, b, "router_wgrad_tc", "router_wgrad_simt"));
   return MOE_OK;
