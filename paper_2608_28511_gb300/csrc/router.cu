@@ -8,62 +8,42 @@
 
 namespace moe {
 
-struct Identity {
-  __device__ __forceinline__ float operator()(float z) const { return z; }
-};
-
-// Four threads per token (select.cuh): the K largest logits, ties to the lower
+// One warp per token (select.cuh): the K largest logits, ties to the lower
 // expert index (reading R2), NaN as -inf, ordered by descending logit.  The
 // probabilities are exp(z_k - z_max) normalised over the K chosen logits,
 // which equals the full softmax renormalised over the chosen set (reading R1).
-template <int KM>
+template <int V>
 __global__ void __launch_bounds__(256) topk_kernel(const float* __restrict__ logits, int64_t T, int E, int K,
-                                                   int tpb, int32_t* __restrict__ idx, float* __restrict__ prob) {
-  extern __shared__ __align__(16) float zs[];  // [tpb][E]
-  const int tid = threadIdx.x;
-  const int64_t t0 = (int64_t)blockIdx.x * tpb;
-  const int n = (int)min((int64_t)tpb, T - t0);
-  sel::stage_rows(logits + t0 * E, zs, n * E, Identity());
-  __syncthreads();
-  const int q = tid >> 2, r = tid & 3;
-  const bool active = q < n;
-  uint64_t win[KM];
-  float unused;
-  sel::quad_topk<KM>(zs + (int64_t)q * E, nullptr, E, K, r, q, active, win, &unused);
-  if (!active) return;
-  const float zmax = sel::unpack_key(win[0]);
-  float w[KM];
-  float sum = 0.f;
+                                                   int32_t* __restrict__ idx, float* __restrict__ prob) {
+  __shared__ uint2 slots[8][kMaxK];
+  const int lane = threadIdx.x & 31;
+  const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (t >= T) return;  // the whole warp
+  const float* row = logits + t * E;
+  float key[V];
 #pragma unroll
-  for (int k = 0; k < KM; ++k) {
-    w[k] = 0.f;
-    if (k < K) {
-      w[k] = expf(sel::unpack_key(win[k]) - zmax);
-      sum += w[k];
-    }
-  }
-  const float inv = 1.0f / sum;
-  const int64_t o = (t0 + q) * K;
-#pragma unroll
-  for (int k = 0; k < KM; ++k) {
-    if (k < K && (k & 3) == r) {
-      idx[o + k] = sel::unpack_e(win[k]);
-      prob[o + k] = w[k] * inv;
-    }
+  for (int v = 0; v < V; ++v)
+    key[v] = v * 32 + lane < E ? sel::key_of(__ldg(row + v * 32 + lane)) : __uint_as_float(sel::kAbsent);
+  float mk, best;
+  int me;
+  sel::warp_topk<V>(key, E, K, lane, slots[threadIdx.x >> 5], [&] { return row; }, &mk, &me, &best);
+  const float w = lane < K ? expf(mk - best) : 0.f;
+  const float inv = 1.0f / sel::sum16(w);
+  if (lane < K) {
+    idx[t * K + lane] = me;
+    prob[t * K + lane] = w * inv;
   }
 }
 
 cudaError_t launch_topk(const Ctx& c, const float* logits, int64_t T, int E, int K, int32_t* idx, float* prob) {
   if (T == 0) return cudaSuccess;
-  const int tpb = sel::tokens_per_block(E);
-  const dim3 grid((unsigned)((T + tpb - 1) / tpb));
-  const size_t smem = (size_t)tpb * E * 4;
+  const unsigned grid = (unsigned)((T + 7) / 8);
   KernelScope ks("topk", c.stream);
-  switch (sel::k_bound(K)) {
-    case 2: topk_kernel<2><<<grid, 4 * tpb, smem, c.stream>>>(logits, T, E, K, tpb, idx, prob); break;
-    case 4: topk_kernel<4><<<grid, 4 * tpb, smem, c.stream>>>(logits, T, E, K, tpb, idx, prob); break;
-    case 8: topk_kernel<8><<<grid, 4 * tpb, smem, c.stream>>>(logits, T, E, K, tpb, idx, prob); break;
-    default: topk_kernel<16><<<grid, 4 * tpb, smem, c.stream>>>(logits, T, E, K, tpb, idx, prob); break;
+  switch (sel::lists_of(E)) {
+    case 1: topk_kernel<1><<<grid, 256, 0, c.stream>>>(logits, T, E, K, idx, prob); break;
+    case 2: topk_kernel<2><<<grid, 256, 0, c.stream>>>(logits, T, E, K, idx, prob); break;
+    case 4: topk_kernel<4><<<grid, 256, 0, c.stream>>>(logits, T, E, K, idx, prob); break;
+    default: topk_kernel<8><<<grid, 256, 0, c.stream>>>(logits, T, E, K, idx, prob); break;
   }
   return cudaGetLastError();
 }

@@ -1,0 +1,43 @@
+"""The warp-per-token top-K selection where its lists are short or ragged and
+where keys are equal, infinite or NaN: indices against a plain sort of the same
+keys (NaN as -inf, -0 as +0, ties to the lower expert)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_28511_gb300 import abi
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("E,K", [(1, 1), (2, 2), (5, 5), (16, 16), (31, 3), (33, 8), (63, 16), (65, 4), (100, 7),
+                                 (129, 9), (255, 16), (256, 1)])
+def test_selection(E, K):
+    T = 333
+    z = torch.randn(T, E, generator=torch.Generator().manual_seed(E * 17 + K))
+    z[0] = float("-inf")                               # every key equal
+    z[1] = 0.0
+    z[1, ::2] = -0.0                                   # -0 ties with +0
+    z[2, : E // 2 + 1] = float("nan")
+    z[3, -1] = float("inf")
+    z[4] = torch.round(z[4])                           # many ties, in and across lists
+    z[5::9] = torch.round(z[5::9] * 2)
+    z[6, :] = z[6, 0]
+    z[6, -1] = float("nan")
+    idx = torch.empty(T, K, dtype=torch.int32, device="cuda")
+    prob = torch.empty(T, K, device="cuda")
+    abi.moe_topk(abi.MoeShape.of(T, 1, K, 64, E, 64), z.cuda(), idx, prob)
+    key = np.where(np.isnan(z.numpy()), -np.inf, z.numpy()) + 0.0
+    ref = np.argsort(-key, axis=1, kind="stable")[:, :K]
+    assert (idx.cpu().numpy() == ref).all()
+    top = np.take_along_axis(key, ref, 1).astype(np.float64)
+    fine = np.isfinite(top[:, 0])                      # an infinite best key has no softmax
+    w = np.exp(top[fine] - top[fine][:, :1])
+    assert np.abs(prob.cpu().numpy()[fine] - w / w.sum(1, keepdims=True)).max() <= 1e-6
+    assert abi.moe_check_device_status() == 0
