@@ -6,7 +6,7 @@
 // records it and drops it.
 //
 // Rounds assume that all chosen keys differ, and the end checks it: one head
-// taken per round, no two taken keys equal, none equal to the last one left.
+// taken per round, no two taken keys equal, none left equal to the last one.
 // Otherwise the token is chosen again by rounds that resolve equal keys to the
 // lower expert.  -0 ties with +0 and NaN keys count as -inf.
 //
@@ -136,7 +136,8 @@ __device__ __forceinline__ void warp_topk(float (&key)[V], int E, int K, int lan
   if (lane < K) r = slot[lane];
   r.y &= 255u;
   const float mine = __uint_as_float(r.x), next = __shfl_down_sync(0xffffffffu, mine, 1);
-  const bool tie = key[0] == m || (lane + 1 < K && mine == next);
+  // m is NaN if the keys ran out, which takes an earlier round that took several
+  const bool tie = key[0] == m || m != m || (lane + 1 < K && mine == next);
   if (__reduce_add_sync(0xffffffffu, (unsigned)taken) != (unsigned)K || __any_sync(0xffffffffu, tie))
     r = topk_with_ties<V>(row(), E, K, lane);
   *my_key = __uint_as_float(r.x);
