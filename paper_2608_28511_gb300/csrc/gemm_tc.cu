@@ -239,6 +239,8 @@ cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name) {
   const int64_t a_inner = pl.a_mn ? d.M : d.K;
   if (!make_map(&p.ta, d.A, a_inner, a_rows, pl.lda * 2, 64, ga ? 1 : (pl.a_mn ? 64 : BM)))
     return cudaErrorInvalidValue;
+  if (d.group == Group::M && !ga && !make_map(&p.ta16, d.A, a_inner, a_rows, pl.lda * 2, 64, tc::kARowStep))
+    return cudaErrorInvalidValue;
   // B: K-major box {64 k, BN / CG n}; MN-major box {64 n, 64 k}
   const int64_t grows = d.group == Group::M ? d.sb_g / pl.ldb : 0;
   int64_t b_rows;
