@@ -88,27 +88,39 @@ __global__ void __launch_bounds__(256) dispatch_fp8_kernel(const uint4* __restri
 }
 
 // x_perm[r] = codes[r] * scale[r] in bf16 (exact), 8 codes (one 16-byte
-// store) per thread step, so a warp writes 512 contiguous bytes.
+// store) per thread step, in the row layout of the NVFP4 receiver.
+template <int L>
 __global__ void __launch_bounds__(256) dequant_rows_kernel(const uint2* __restrict__ xq,
                                                            const float* __restrict__ scale, int64_t rows, int vpr,
                                                            uint4* __restrict__ out) {
-  const int64_t total = rows * vpr;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const float s = __ldg(scale + i / vpr);
-    const uint2 q = __ldg(xq + i);
-    const uint32_t w[2] = {q.x, q.y};
-    float f[8];
+  constexpr int U = 4;
+  const int64_t r = (int64_t)blockIdx.x * (256 / L) + threadIdx.x / L;
+  if (r >= rows) return;
+  xq += r * vpr;
+  out += r * vpr;
+  const float s = __ldg(scale + r);
+  for (int v0 = threadIdx.x % L; v0 < vpr; v0 += U * L) {
+    uint2 q[U];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int u = 0; u < U; ++u) q[u] = v0 + u * L < vpr ? __ldcs(xq + v0 + u * L) : make_uint2(0u, 0u);
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(w[h] >> (16 * j)), __NV_E4M3);
-        const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&hr));
-        f[4 * h + 2 * j] = v.x * s;
-        f[4 * h + 2 * j + 1] = v.y * s;
+    for (int u = 0; u < U; ++u) {
+      const int v = v0 + u * L;
+      if (v >= vpr) break;
+      const uint32_t w[2] = {q[u].x, q[u].y};
+      float f[8];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(w[h] >> (16 * j)), __NV_E4M3);
+          const float2 p = __half22float2(*reinterpret_cast<const __half2*>(&hr));
+          f[4 * h + 2 * j] = p.x * s;
+          f[4 * h + 2 * j + 1] = p.y * s;
+        }
       }
+      st_stream(out + v, pack16<bf16>(f));
     }
-    st_stream(out + i, pack16<bf16>(f));
   }
 }
 
@@ -139,10 +151,14 @@ cudaError_t launch_dispatch_fp8(const Ctx& c, const void* x, const int32_t* row_
 cudaError_t launch_dequant_rows(const Ctx& c, const void* xq, const float* scale, int64_t rows, int D, void* out) {
   if (rows == 0) return cudaSuccess;
   const int vpr = D / 8;
-  const int64_t want = (rows * vpr + 255) / 256;
-  const int blocks = (int)(want < (int64_t)c.num_sms * 16 ? want : (int64_t)c.num_sms * 16);
+  const int L = vpr >= 32 ? 32 : vpr >= 16 ? 16 : 8;
+  const int rpb = 256 / L;
+  const unsigned blocks = (unsigned)((rows + rpb - 1) / rpb);
+  const uint2* q = (const uint2*)xq;
   KernelScope ks("dequant_rows", c.stream);
-  dequant_rows_kernel<<<blocks, 256, 0, c.stream>>>((const uint2*)xq, scale, rows, vpr, (uint4*)out);
+  if (L == 32) dequant_rows_kernel<32><<<blocks, 256, 0, c.stream>>>(q, scale, rows, vpr, (uint4*)out);
+  else if (L == 16) dequant_rows_kernel<16><<<blocks, 256, 0, c.stream>>>(q, scale, rows, vpr, (uint4*)out);
+  else dequant_rows_kernel<8><<<blocks, 256, 0, c.stream>>>(q, scale, rows, vpr, (uint4*)out);
   return cudaGetLastError();
 }
 
