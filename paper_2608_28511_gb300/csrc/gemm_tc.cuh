@@ -5,7 +5,7 @@
 // CTA per SM walks a static tile sequence decoded on the device from the
 // expert offsets (no host synchronisation).  Warp roles:
 //   warp 0      TMA producer (one lane) filling a kStages-deep smem ring;
-//   warp 1      TMEM allocator and MMA issuer (one lane issues, all wait);
+//   warp 1      TMEM allocator and MMA issuer (one lane);
 //   warps 2..   epilogue (4, or 8 for bf16 outputs): TMEM -> registers ->
 //               global, one accumulator row per thread, double-buffered
 //               accumulators (2 x BN columns);
@@ -36,6 +36,7 @@ namespace tc {
 constexpr int BM = 128;
 constexpr int BK = 64;                  // bf16: 128 bytes, one swizzle row
 constexpr uint64_t kWaitLimitNs = 4000000000ull;
+constexpr uint32_t kSuspendNs = 20000;  // a try sleeps up to this long for its phase
 
 struct Params {
   CUtensorMap ta;
@@ -93,10 +94,10 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}\n"
       : "=r"(ok)
-      : "r"(bar), "r"(parity)
+      : "r"(bar), "r"(parity), "r"(kSuspendNs)
       : "memory");
   return ok != 0;
 }
@@ -112,6 +113,18 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
       : "=r"(ok)
       : "r"(bar), "r"(parity)
       : "memory");
+  return ok != 0;
+}
+// One lane of a converged warp.  TMA copies, MMAs and commits are issued under
+// it and not under a lane comparison: their operands have to be uniform, which
+// only this predicate tells the compiler.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(ok));
   return ok != 0;
 }
 __device__ __forceinline__ uint64_t global_timer_ns() {
@@ -952,7 +965,7 @@ __global__ void __launch_bounds__(
     }
   } else if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       int issued = 0;
@@ -1044,51 +1057,56 @@ __global__ void __launch_bounds__(
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (the leader CTA)
-    int stage = 0;
-    uint32_t phase = 0;
-    int acc = 0;
-    uint32_t acc_phase = 0;
-    bool ok = true;
-    bool issued_any = false;
+    // One lane runs the whole loop.  What bounds it is how fast one thread issues
+    // a k-block's four MMAs: with all lanes looping and lane 0 issuing, 0.31 us
+    // per k-block at any tile size (MMAs of 256 x 256 take 0.27), now 0.13.
+    // At T = 8192, D = 2048, E = 64, K = 6, F = 1024: GEMM-1 289 -> 272 us, GEMM-2
+    // 147 -> 141, their dgrads 277 -> 262 and 179 -> 172.
     constexpr uint16_t kBoth = 0x3;
-    Walker wk = make_walker<GROUP>(cta0, ncta, total, kper, knce, knz, ktot, ksnake);
-    for (int t; ok && leader && next_tile<GROUP>(wk, s_off, s_pref, t);) {
-      Tile ti;
-      decode_tile<GROUP, CG>(p, t, s_off, s_pref, rank, ti);
-      if (ti.nkb == 0) continue;
-      issued_any = true;
-      if (!wait_bounded(smem_u32(&tempty[acc]), acc_phase ^ 1u, &s_abort, p.err)) { ok = false; break; }
-      tc_fence_after();
-      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-      for (int kb = 0; kb < ti.nkb; ++kb) {
-        if (!wait_bounded(smem_u32(&full[stage]), phase, &s_abort, p.err, GATHER != 0 && CG == 2)) {
-          ok = false;
-          break;
-        }
-        if (GATHER != 0) fence_proxy_async_smem();  // the row copies, before the tensor core reads them
+    if (leader && elect_one()) {
+      int stage = 0;
+      uint32_t phase = 0;
+      int acc = 0;
+      uint32_t acc_phase = 0;
+      bool ok = true;
+      bool issued_any = false;
+      Walker wk = make_walker<GROUP>(cta0, ncta, total, kper, knce, knz, ktot, ksnake);
+      for (int t; ok && next_tile<GROUP>(wk, s_off, s_pref, t);) {
+        Tile ti;
+        decode_tile<GROUP, CG>(p, t, s_off, s_pref, rank, ti);
+        if (ti.nkb == 0) continue;
+        issued_any = true;
+        if (!wait_bounded(smem_u32(&tempty[acc]), acc_phase ^ 1u, &s_abort, p.err)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t sa = smem_u32(smem + stage * C::kStageBytes);
-        const uint32_t sb = sa + C::kABytes;
-        if (lane == 0) {
-#pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            uint64_t ad, bd;
-            if (A_MN) ad = make_sdesc(sa + k * 2048, 8192, 1024);
-            else ad = make_sdesc(sa + k * 32, 16, 1024);
-            if (B_MN) bd = make_sdesc(sb + k * 2048, 8192, 1024);
-            else bd = make_sdesc(sb + k * 32, 16, 1024);
-            mma_bf16_cg<CG>(d_tmem, ad, bd, kIdesc, (kb > 0 || k > 0) ? 1u : 0u);
+        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+        for (int kb = 0; kb < ti.nkb; ++kb) {
+          if (!wait_bounded(smem_u32(&full[stage]), phase, &s_abort, p.err, GATHER != 0 && CG == 2)) {
+            ok = false;
+            break;
           }
+          if (GATHER != 0) fence_proxy_async_smem();  // the row copies, before the tensor core reads them
+          tc_fence_after();
+          const uint32_t sa = smem_u32(smem + stage * C::kStageBytes);
+          const uint64_t ad = make_sdesc(sa, A_MN ? 8192 : 16, 1024);
+          const uint64_t bd = make_sdesc(sa + C::kABytes, B_MN ? 8192 : 16, 1024);
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k)  // 16 elements of k: 32 bytes, or 2048 MN-major, in units of 16
+            mma_bf16_cg<CG>(d_tmem, ad + k * (A_MN ? 128 : 2), bd + k * (B_MN ? 128 : 2), kIdesc,
+                            (kb > 0 || k > 0) ? 1u : 0u);
           mma_commit_cg<CG>(smem_u32(&empty[stage]), kBoth);
+          if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
         }
-        __syncwarp();
-        if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
+        if (!ok) break;
+        mma_commit_cg<CG>(smem_u32(&tfull[acc]), kBoth);
+        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
-      if (!ok) break;
-      if (lane == 0) mma_commit_cg<CG>(smem_u32(&tfull[acc]), kBoth);
-      __syncwarp();
-      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+      // drain: all MMAs issued have completed before TMEM is freed
+      if (issued_any) {
+        mma_commit_cg<CG>(smem_u32(done), 0x1);
+        wait_drain(smem_u32(done), 0, 1000000000ull);
+      }
     }
+    __syncwarp();
     if (GATHER != 0 && CG == 2 && !leader && lane == 0) {
       // the other CTA of a pair: forward each stage whose row copies have all
       // landed here (this CTA's full barrier) to the leader's full barrier
@@ -1106,11 +1124,6 @@ __global__ void __launch_bounds__(
           if (++fs == C::kStages) { fs = 0; fph ^= 1u; }
         }
       }
-    }
-    // drain: all MMAs issued by this warp have completed before TMEM is freed
-    if (lane == 0 && issued_any) {
-      mma_commit_cg<CG>(smem_u32(done), 0x1);
-      wait_drain(smem_u32(done), 0, 1000000000ull);
     }
     __syncwarp();
   } else if (kZW && warp == 2 + EW) {
