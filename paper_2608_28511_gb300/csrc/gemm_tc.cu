@@ -125,10 +125,26 @@ bool make_plan(const GemmDesc& d, Plan* pl) {
   pl->cg = 1;
   if (d.group == Group::Dense && d.epi == Epi::StoreBias) {
     pl->bn = d.N <= 64 ? 64 : (d.N <= 128 ? 128 : 256);  // router logits: N = E
+    pl->cg = 2;
   } else if (d.group == Group::M || d.M > BM) {
     pl->cg = 2;
   }
   return true;
+}
+
+// Rows per CTA of a router-logit tile (N = E fits one column tile, so tiles are
+// rows only).  The GEMM is bound by the copies into each SM, so every SM gets
+// an equal share: the tiles of n full-height rounds over the pairs are cut down
+// to one height, in whole 8-row swizzle atoms.  With 128-row tiles on single
+// CTAs a batch of 8192 ran on 64 SMs and one of 30011 took two uneven rounds,
+// and every tile copied all of W_r; a pair's CTAs copy half each.  T = 30011,
+// E = 128, D = 2048 (139 MB): 27.0 -> 24.1 us; T = 2045, E = 60: 10.7 -> 9.7;
+// T = 16384, E = 256, 4096 wide: 36 -> 31; T = 8192, E = 64: 10.9 -> 11.7.
+int router_tile_rows(int64_t M, int num_sms) {
+  const int64_t slots = num_sms / 2 * 2;
+  const int64_t rounds = (M + slots * BM - 1) / (slots * BM);
+  const int64_t rows = (M + rounds * slots - 1) / (rounds * slots);
+  return (int)((rows + 7) / 8 * 8);
 }
 
 // Co-resident 2-CTA clusters of an instantiation (0 if the query fails).
@@ -230,14 +246,15 @@ cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name) {
   if (!make_plan(d, &pl) || !gemm_tc_supports(d)) return cudaErrorNotSupported;
   Params p;
   memset(&p, 0, sizeof(p));
-  const int bn = pl.bn, bmp = BM * pl.cg, bnc = bn / pl.cg;
+  p.tile_rows = d.group == Group::Dense && d.epi == Epi::StoreBias ? router_tile_rows(d.M, c.num_sms) : BM;
+  const int bn = pl.bn, bmp = p.tile_rows * pl.cg, bnc = bn / pl.cg;
   // A: K-major box {64 k, 128 m}; MN-major box {64 m, 64 k}
   const bool ga = d.gather && d.group == Group::M;  // A's rows gathered (cp.async row copies; its map unused)
   const bool gb = d.gather && d.group == Group::K;  // B's k rows gathered (cp.async row copies; its map unused)
   int64_t a_rows = pl.a_mn ? (d.group == Group::K ? d.max_rows : d.K) : (d.group == Group::M ? d.max_rows : d.M);
   if (ga) a_rows = d.gather_rows;
   const int64_t a_inner = pl.a_mn ? d.M : d.K;
-  if (!make_map(&p.ta, d.A, a_inner, a_rows, pl.lda * 2, 64, ga ? 1 : (pl.a_mn ? 64 : BM)))
+  if (!make_map(&p.ta, d.A, a_inner, a_rows, pl.lda * 2, 64, ga ? 1 : (pl.a_mn ? 64 : p.tile_rows)))
     return cudaErrorInvalidValue;
   if (d.group == Group::M && !ga && !make_map(&p.ta16, d.A, a_inner, a_rows, pl.lda * 2, 64, tc::kARowStep))
     return cudaErrorInvalidValue;
@@ -302,6 +319,11 @@ cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name) {
   if (ga) return launch_inst<256, false, false, 1, 3, bf16, 2, 1>(c, p, ub);
   if (gb && pl.cg == 2) return launch_inst<256, true, true, 2, 0, float, 2, 2>(c, p, ub);
   if (gb) return launch_inst<256, true, true, 2, 0, float, 1, 2>(c, p, ub);
+  if (g == 0 && e == 1) {
+    if (bn == 64) return launch_inst<64, false, false, 0, 1, float, 2>(c, p, ub);
+    if (bn == 128) return launch_inst<128, false, false, 0, 1, float, 2>(c, p, ub);
+    return launch_inst<256, false, false, 0, 1, float, 2>(c, p, ub);
+  }
   if (pl.cg == 2) {
     if (g == 2) return launch_inst<256, true, true, 2, 0, float, 2>(c, p, ub);
     if (g == 1 && !pl.b_mn && e == 3) return launch_inst<256, false, false, 1, 3, bf16, 2>(c, p, ub);
@@ -317,11 +339,6 @@ cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name) {
     return cudaErrorNotSupported;
   }
   if (g == 2) return launch_inst<256, true, true, 2, 0, float, 1>(c, p, ub);
-  if (g == 0 && e == 1) {
-    if (bn == 64) return launch_inst<64, false, false, 0, 1, float, 1>(c, p, ub);
-    if (bn == 128) return launch_inst<128, false, false, 0, 1, float, 1>(c, p, ub);
-    return launch_inst<256, false, false, 0, 1, float, 1>(c, p, ub);
-  }
   if (g == 0 && !pl.a_mn && !pl.b_mn && e == 0) return launch_inst<256, false, false, 0, 0, bf16, 1>(c, p, ub);
   if (g == 0 && !pl.a_mn && !pl.b_mn && e == 2) return launch_inst<256, false, false, 0, 2, bf16, 1>(c, p, ub);
   if (g == 0 && !pl.a_mn && !pl.b_mn && e == 4) return launch_inst<256, false, false, 0, 4, bf16, 1>(c, p, ub);

@@ -46,6 +46,7 @@ struct Params {
   int64_t b_group_rows;   // rows of B's tensor map per group (Group::M)
   int num_groups;
   int tiles_m, tiles_n;
+  int tile_rows;          // Dense: rows of a tile per CTA (BM, or fewer with a K-major A)
   const int32_t* offsets;
   void* C;
   int64_t ldc, sc_g;
@@ -511,8 +512,8 @@ __device__ __forceinline__ void decode_tile(const Params& p, int t, const int* s
   if (GROUP == 0) {
     const int mt = t / p.tiles_n, nt = t % p.tiles_n;
     ti.g = 0;
-    ti.row0 = (int64_t)mt * BMP + rank * BM;
-    ti.row_end = p.M;
+    ti.row0 = ((int64_t)mt * CG + rank) * p.tile_rows;
+    ti.row_end = p.M < ti.row0 + p.tile_rows ? p.M : ti.row0 + p.tile_rows;
     ti.n0 = nt;
     ti.kbeg = 0;
     ti.kend = p.K;
@@ -977,9 +978,9 @@ __global__ void __launch_bounds__(
         decode_tile<GROUP, CG>(p, t, s_off, s_pref, rank, ti);
         const int64_t nb = ti.n0 * BN + (int64_t)rank * BNC;  // this CTA's first B row / column
         // Group::M: the A rows that exist (kAShort); the leader expects both CTAs' copies
-        const int arows = GROUP == 1 ? a_rows_copied(ti.row0, ti.row_end) : BM;
+        const int arows = GROUP == 1 ? a_rows_copied(ti.row0, ti.row_end) : GROUP == 0 ? p.tile_rows : BM;
         const int abytes =
-            (GROUP == 1 ? arows + (CG == 2 ? a_rows_copied(ti.row0 + BM, ti.row_end) : 0) : CG * BM) * BK * 2;
+            (GROUP == 1 ? arows + (CG == 2 ? a_rows_copied(ti.row0 + BM, ti.row_end) : 0) : CG * arows) * BK * 2;
         for (int kb = 0; kb < ti.nkb; ++kb) {
           if (!wait_bounded(smem_u32(&empty[stage]), phase ^ 1u, &s_abort, p.err)) { ok = false; break; }
           const uint32_t fb_local = smem_u32(&full[stage]);
@@ -1016,7 +1017,7 @@ __global__ void __launch_bounds__(
             if (A_MN) {
               load(sa, &p.ta, (int)ti.row0, k0);
               load(sa + 8192, &p.ta, (int)ti.row0 + 64, k0);
-            } else if (arows == BM) {
+            } else if (GROUP == 0 || arows == BM) {
               load(sa, &p.ta, k0, (int)ti.row0);
             } else {
               for (int r = 0; r < arows; r += kARowStep) load(sa + r * BK * 2, &p.ta16, k0, (int)ti.row0 + r);
@@ -1404,15 +1405,15 @@ __global__ void __launch_bounds__(
           if (col0 >= p.N) break;
           tmem_ld32(tbase + c * 32, v);
           const int nvalid = (int)imin64(32, p.N - col0);
-          if (EPI == 1 || nvalid < 32) {
-            // router logits (E columns, possibly ragged): direct row stores
+          if (EPI == 1 && p.bias) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              if (i < nvalid) v[i] += p.bias[col0 + i];
+          }
+          if (nvalid < 32) {
+            // ragged columns: direct row stores
             if (!vrow) continue;
             TC* crow = Cb + grow * p.ldc;
-            if (EPI == 1 && p.bias) {
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (i < nvalid) v[i] += p.bias[col0 + i];
-            }
             if (EPI == 2) {
 #pragma unroll
               for (int i = 0; i < 32; ++i)
@@ -1424,7 +1425,7 @@ __global__ void __launch_bounds__(
               for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i], 0.f) * fmaxf(v[i], 0.f);
               store_row32<TC>(static_cast<TC*>(p.aux) + grow * p.ldc + col0, v, nvalid);
             }
-          } else if (EPI == 0 || EPI == 4) {
+          } else if (EPI == 0 || EPI == 1 || EPI == 4) {
 #pragma unroll
             for (int r = 0; r < RPC; ++r) {
 #pragma unroll
