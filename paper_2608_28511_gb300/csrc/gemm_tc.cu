@@ -170,12 +170,12 @@ int max_pair_clusters(KernelT k, int smem, int threads) {
 }
 
 // ub = upper bound on the number of tiles (each tile is one CTA, or one pair for CG 2).
-template <int BN, bool A_MN, bool B_MN, int GROUP, int EPI, typename TC, int CG, int GATHER = 0>
+template <int BN, bool A_MN, bool B_MN, int GROUP, int EPI, typename TC, int CG, int GATHER = 0, int EWF = 4>
 cudaError_t launch_inst(const Ctx& c, const Params& p, int64_t ub) {
-  auto k = tc::gemm_tc_kernel<BN, A_MN, B_MN, GROUP, EPI, TC, CG, GATHER>;
+  auto k = tc::gemm_tc_kernel<BN, A_MN, B_MN, GROUP, EPI, TC, CG, GATHER, EWF>;
   constexpr int kZW = (GROUP == 2 && sizeof(TC) == 4 && GATHER == 0) ? 1 : 0;
-  constexpr int kSmem = Cfg<BN, CG, sizeof(TC), EPI, kZW>::kSmem;
-  constexpr int kThreads = Cfg<BN, CG, sizeof(TC), EPI, kZW>::kThreads;
+  constexpr int kSmem = Cfg<BN, CG, sizeof(TC), EPI, kZW, EWF>::kSmem;
+  constexpr int kThreads = Cfg<BN, CG, sizeof(TC), EPI, kZW, EWF>::kThreads;
   static bool configured = false;
   static int pairs = 0;
   if (!configured) {
@@ -325,7 +325,16 @@ cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name) {
     return launch_inst<256, false, false, 0, 1, float, 2>(c, p, ub);
   }
   if (pl.cg == 2) {
-    if (g == 2) return launch_inst<256, true, true, 2, 0, float, 2>(c, p, ub);
+    if (g == 2) {
+      // short groups (up to ten k-blocks a tile on average): eight epilogue warps.
+      // GEMM-2's and GEMM-1's weight gradient, four warps -> eight: 136 rows per
+      // expert, D = 2048, F = 1408, E = 60: 154 -> 140 and 273 -> 243 us; 512 rows
+      // (D = 1024, F = 768, E = 256) 204 -> 201 and 373 -> 373; 768 rows (D = 2048,
+      // F = 1024, E = 64) 157 -> 160 and 299 -> 305.
+      if (d.offsets && d.max_rows <= 10 * (int64_t)tc::BK * d.num_groups)
+        return launch_inst<256, true, true, 2, 0, float, 2, 0, 8>(c, p, ub);
+      return launch_inst<256, true, true, 2, 0, float, 2>(c, p, ub);
+    }
     if (g == 1 && !pl.b_mn && e == 3) return launch_inst<256, false, false, 1, 3, bf16, 2>(c, p, ub);
     if (g == 1 && !pl.b_mn && e == 0) return launch_inst<256, false, false, 1, 0, bf16, 2>(c, p, ub);
     if (g == 1 && pl.b_mn && e == 0) return launch_inst<256, false, true, 1, 0, bf16, 2>(c, p, ub);

@@ -6,7 +6,7 @@
 // expert offsets (no host synchronisation).  Warp roles:
 //   warp 0      TMA producer (one lane) filling a kStages-deep smem ring;
 //   warp 1      TMEM allocator and MMA issuer (one lane);
-//   warps 2..   epilogue (4, or 8 for bf16 outputs): TMEM -> registers ->
+//   warps 2..   epilogue (4 or 8): TMEM -> registers ->
 //               global, one accumulator row per thread, double-buffered
 //               accumulators (2 x BN columns);
 //   last warp   Group::K with fp32 gradients only: writes the empty groups'
@@ -393,7 +393,7 @@ __host__ __device__ constexpr uint32_t make_idesc(int bn, int bm, bool a_mn, boo
 // CG = 1: one CTA computes a 128 x BN tile.  CG = 2: a cluster of two CTAs
 // computes a 256 x BN tile; each CTA stages its 128 rows of A and BN / 2 rows
 // of B, and holds its 128 accumulator rows in its own TMEM.
-template <int BN, int CG = 1, int TCB = 2, int EPI = 0, int ZW = 0>  // TCB: bytes per element of C
+template <int BN, int CG = 1, int TCB = 2, int EPI = 0, int ZW = 0, int EWF = 4>  // TCB: bytes per element of C
 struct Cfg {
   static constexpr int kBRows = BN / CG;
   static constexpr int kABytes = BM * BK * 2;
@@ -403,18 +403,20 @@ struct Cfg {
   static constexpr int kStages = EPI == 5 ? 5 : ((196608 / kStageBytes) < 8 ? (196608 / kStageBytes) : 8);
   static constexpr int kCols = 2 * BN;  // double-buffered fp32 accumulator
   // Epilogue warps: 8 (two per TMEM lane quarter, each taking half the
-  // columns) for bf16 outputs, whose epilogues are latency-bound; 4 for fp32
-  // outputs, which are bound by their store bandwidth.
-  static constexpr int kEpiWarps = TCB == 2 ? 8 : 4;
+  // columns) for bf16 outputs, whose epilogues are latency-bound; EWF for fp32
+  // outputs: 4, which are bound by their store bandwidth beside a long main
+  // loop, or 8 where a tile has few k-blocks and its stores are what it takes.
+  static constexpr int kEpiWarps = TCB == 2 ? 8 : EWF;
   // ZW: one more warp that writes the empty groups' zero gradients (Group::K, fp32)
   static constexpr int kThreads = 64 + 32 * kEpiWarps + 32 * ZW;
   // per epilogue warp: 32 rows x 32 columns of C staging, rows padded by 16 B
-  // (conflict-free both ways)
+  // (conflict-free both ways); eight warps of fp32 rows stage 16 rows at a time
+  static constexpr int kStageRows = TCB == 4 && kEpiWarps == 8 ? 16 : 32;
   static constexpr int kRowBytes = 32 * TCB;
   static constexpr int kPitch = kRowBytes + 16;
   // EPI 5: a ring of three 2 KB slots per warp, each the gate and up blocks of
   // h (in) and of dH (out) for 16 columns of dA, 32 rows x 32 bytes apiece
-  static constexpr int kStageBufBytes = EPI == 5 ? 6144 : 32 * kPitch;
+  static constexpr int kStageBufBytes = EPI == 5 ? 6144 : kStageRows * kPitch;
   static constexpr int kStagingBytes = kEpiWarps * kStageBufBytes;
   static constexpr int kSmem = kStages * kStageBytes + kStagingBytes + 1024 /*align*/ + 512 /*barriers*/;
 };
@@ -447,6 +449,25 @@ __device__ __forceinline__ void stage_store(const uint8_t* buf, int lane, uint8_
     const int r = it * RPI + lane / CPR, c = lane % CPR;
     const uint4 v = *reinterpret_cast<const uint4*>(buf + r * (NB + 16) + c * 16);
     if (r < nrows) *reinterpret_cast<uint4*>(gbase + r * ld_bytes + c * 16) = v;
+  }
+}
+// A row of NB bytes per lane -> gbase + lane * ld_bytes through buf, RS rows at
+// a time (rows >= nrows are skipped).
+template <int NB, int RS>
+__device__ __forceinline__ void stage_rows(uint8_t* buf, int lane, const uint4* row, uint8_t* gbase,
+                                           int64_t ld_bytes, int nrows) {
+  constexpr int CPR = NB / 16, RPI = 32 / CPR;
+#pragma unroll
+  for (int r0 = 0; r0 < 32; r0 += RS) {
+    __syncwarp();
+    if (RS == 32 || lane / RS == r0 / RS) stage_put<NB>(buf, lane % RS, row);
+    __syncwarp();
+#pragma unroll
+    for (int it = 0; it < RS / RPI; ++it) {
+      const int r = it * RPI + lane / CPR, c = lane % CPR;
+      const uint4 v = *reinterpret_cast<const uint4*>(buf + r * (NB + 16) + c * 16);
+      if (r0 + r < nrows) *reinterpret_cast<uint4*>(gbase + (r0 + r) * ld_bytes + c * 16) = v;
+    }
   }
 }
 // The 32 x 32 bf16 block of C an accumulating chunk adds to, fetched into
@@ -669,12 +690,12 @@ __device__ __forceinline__ void load_row32(const T* src, float* v) {
 // GATHER: 0 tiled copies; 1 A's rows (K-major, Group::M) and 2 B's k rows
 // (MN-major, Group::K) are gathered from a source matrix through p.gather
 // (row -> source row), four rows per copy, by the 32 lanes of the producer warp.
-template <int BN, bool A_MN, bool B_MN, int GROUP, int EPI, typename TC, int CG, int GATHER = 0>
+template <int BN, bool A_MN, bool B_MN, int GROUP, int EPI, typename TC, int CG, int GATHER = 0, int EWF = 4>
 __global__ void __launch_bounds__(
-    Cfg<BN, CG, sizeof(TC), 0, (GROUP == 2 && sizeof(TC) == 4 && GATHER == 0) ? 1 : 0>::kThreads, 1)
+    Cfg<BN, CG, sizeof(TC), 0, (GROUP == 2 && sizeof(TC) == 4 && GATHER == 0) ? 1 : 0, EWF>::kThreads, 1)
     gemm_tc_kernel(const __grid_constant__ Params p) {
   constexpr int kZW = (GROUP == 2 && sizeof(TC) == 4 && GATHER == 0) ? 1 : 0;  // the zero-gradient warp
-  using C = Cfg<BN, CG, sizeof(TC), EPI, kZW>;
+  using C = Cfg<BN, CG, sizeof(TC), EPI, kZW, EWF>;
   constexpr int EW = C::kEpiWarps;
   constexpr int CSTEP = EW / 4;  // epilogue warps sharing a lane quarter
   constexpr int BMP = BM * CG;
@@ -1209,10 +1230,7 @@ __global__ void __launch_bounds__(
           if (p.N - col0 >= 32) {
 #pragma unroll
             for (int r = 0; r < RPC; ++r) {
-              __syncwarp();
-              stage_put<RB>(stg, lane, z);
-              __syncwarp();
-              stage_store<RB>(stg, lane, c_rows + (col0 + r * CPR) * sizeof(TC), ldc_b, nrows);
+              stage_rows<RB, C::kStageRows>(stg, lane, z, c_rows + (col0 + r * CPR) * sizeof(TC), ldc_b, nrows);
             }
           } else if (vrow) {
             float zf[32];
@@ -1275,24 +1293,15 @@ __global__ void __launch_bounds__(
             tmem_ld32(tbase + blk * 128 + 64 + half * 32, u);
 #pragma unroll
             for (int i = 0; i < NP; ++i) pk[i] = pack16<TC>(v + i * Vec<TC>::N);
-            __syncwarp();
-            stage_put<RB>(stg, lane, pk);
-            __syncwarp();
-            stage_store<RB>(stg, lane, c_rows + (cb + half * 32) * sizeof(TC), ldc_b, nrows);
+            stage_rows<RB, C::kStageRows>(stg, lane, pk, c_rows + (cb + half * 32) * sizeof(TC), ldc_b, nrows);
 #pragma unroll
             for (int i = 0; i < NP; ++i) pk[i] = pack16<TC>(u + i * Vec<TC>::N);
-            __syncwarp();
-            stage_put<RB>(stg, lane, pk);
-            __syncwarp();
-            stage_store<RB>(stg, lane, c_rows + (cb + 64 + half * 32) * sizeof(TC), ldc_b, nrows);
+            stage_rows<RB, C::kStageRows>(stg, lane, pk, c_rows + (cb + 64 + half * 32) * sizeof(TC), ldc_b, nrows);
 #pragma unroll
             for (int i = 0; i < 32; ++i) v[i] = silu_f(v[i]) * u[i];
 #pragma unroll
             for (int i = 0; i < NP; ++i) pk[i] = pack16<TC>(v + i * Vec<TC>::N);
-            __syncwarp();
-            stage_put<RB>(stg, lane, pk);
-            __syncwarp();
-            stage_store<RB>(stg, lane, a_rows + (cb / 2 + half * 32) * sizeof(TC), lda_b, nrows);
+            stage_rows<RB, C::kStageRows>(stg, lane, pk, a_rows + (cb / 2 + half * 32) * sizeof(TC), lda_b, nrows);
           }
         }
       } else if (EPI == 5) {
@@ -1383,10 +1392,7 @@ __global__ void __launch_bounds__(
           for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 #pragma unroll
           for (int j = 0; j < NP; ++j) pk[j] = pack16<TC>(v + j * Vec<TC>::N);
-          __syncwarp();
-          stage_put<RB>(stg, lane, pk);
-          __syncwarp();
-          stage_store<RB>(stg, lane, c_rows + (n0 + (ch + i * CSTEP) * 32) * sizeof(TC), ldc_b, nrows);
+          stage_rows<RB, C::kStageRows>(stg, lane, pk, c_rows + (n0 + (ch + i * CSTEP) * 32) * sizeof(TC), ldc_b, nrows);
         };
         tmem_ld32_issue(tbase + ch * 32, ra);
 #pragma unroll 1
@@ -1430,10 +1436,7 @@ __global__ void __launch_bounds__(
             for (int r = 0; r < RPC; ++r) {
 #pragma unroll
               for (int i = 0; i < NP; ++i) pk[i] = pack16<TC>(v + r * CPR + i * Vec<TC>::N);
-              __syncwarp();
-              stage_put<RB>(stg, lane, pk);
-              __syncwarp();
-              stage_store<RB>(stg, lane, c_rows + (col0 + r * CPR) * sizeof(TC), ldc_b, nrows);
+              stage_rows<RB, C::kStageRows>(stg, lane, pk, c_rows + (col0 + r * CPR) * sizeof(TC), ldc_b, nrows);
             }
             if (EPI == 4) {
               // a = relu(h)^2 at the same positions of aux
@@ -1444,10 +1447,7 @@ __global__ void __launch_bounds__(
               for (int r = 0; r < RPC; ++r) {
 #pragma unroll
                 for (int i = 0; i < NP; ++i) pk[i] = pack16<TC>(v + r * CPR + i * Vec<TC>::N);
-                __syncwarp();
-                stage_put<RB>(stg, lane, pk);
-                __syncwarp();
-                stage_store<RB>(stg, lane, a_rows + (col0 + r * CPR) * sizeof(TC), ldc_b, nrows);
+                stage_rows<RB, C::kStageRows>(stg, lane, pk, a_rows + (col0 + r * CPR) * sizeof(TC), ldc_b, nrows);
               }
             }
           }
