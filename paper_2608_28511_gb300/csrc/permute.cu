@@ -184,18 +184,43 @@ static inline int k_bound(int K) { return K <= 2 ? 2 : (K <= 4 ? 4 : (K <= 8 ? 8
     default: { constexpr int KM = 16; CALL; break; } \
   }
 
+// Warps per token (P): a warp walks its row 32 vectors at a time, and each step
+// is a round trip to memory, so a batch with few rows is bound by that chain.
+// Eight warps share a token's row where fewer than 16 rows per SM are in flight
+// with one warp per token: T = 64, K = 6, D = 2048 dispatch 8.6 -> 3.6 us,
+// combine 9.6 -> 4.1.  Above it is even (8180 rows of 4 KB) or slower (9003 rows
+// of 2 KB: fused dispatch / router backward 8 -> 16 us).
+static inline int row_parts(const Ctx& c, int64_t T, int K, int vpr) {
+  return vpr >= 128 && T * K < (int64_t)c.num_sms * 16 ? 8 : 1;
+}
+// Token and part of this warp: the parts of a token are consecutive warps of one
+// block of 8.
+struct WarpToken {
+  int64_t t;
+  int part;
+};
+template <int P>
+__device__ __forceinline__ WarpToken warp_token() {
+  const int w = threadIdx.x >> 5;
+  return {((int64_t)blockIdx.x * 8 + w) / P, w % P};
+}
+static inline unsigned row_grid(int64_t T, int P) { return (unsigned)((T * P + 7) / 8); }
+#define MOE_DISPATCH_KM_P(K, parts, CALL)                                  \
+  if ((parts) == 1) { constexpr int P = 1; MOE_DISPATCH_KM(K, CALL) }      \
+  else { constexpr int P = 8; MOE_DISPATCH_KM(K, CALL) }
+
 // Dispatch: each token's row is read once and written to its K rows.
-template <int KM>
+template <int KM, int P>
 __global__ void __launch_bounds__(256) dispatch_rows_kernel(const uint4* __restrict__ x,
                                                             const int32_t* __restrict__ row_of_slot, int64_t T,
                                                             int K, int vpr, uint4* __restrict__ x_perm) {
   const int lane = threadIdx.x & 31;
-  const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const auto [t, part] = warp_token<P>();
   if (t >= T) return;
   int32_t rows[KM];
   load_rows<KM>(row_of_slot, t, K, rows);
   const uint4* src = x + t * vpr;
-  for (int v = lane; v < vpr; v += 32) {
+  for (int v = part * 32 + lane; v < vpr; v += 32 * P) {
     const uint4 val = ld_stream(src + v);
 #pragma unroll
     for (int k = 0; k < KM; ++k)
@@ -207,30 +232,31 @@ cudaError_t launch_dispatch_rows(const Ctx& c, const void* x, const int32_t* row
                                  int64_t row_bytes, void* x_perm) {
   if (T == 0) return cudaSuccess;
   const int warps = 8;
-  const unsigned grid = (unsigned)((T + warps - 1) / warps);
   const int vpr = (int)(row_bytes / 16);
+  const int parts = row_parts(c, T, K, vpr);
+  const unsigned grid = row_grid(T, parts);
   KernelScope ks("dispatch_rows", c.stream);
-  MOE_DISPATCH_KM(K, (dispatch_rows_kernel<KM><<<grid, 32 * warps, 0, c.stream>>>(
+  MOE_DISPATCH_KM_P(K, parts, (dispatch_rows_kernel<KM, P><<<grid, 32 * warps, 0, c.stream>>>(
                          (const uint4*)x, row_of_slot, T, K, vpr, (uint4*)x_perm)));
   return cudaGetLastError();
 }
 
 // Combine: y[t] = sum_k p_k Y_perm[row_k], fp32 accumulation, one rounding.
-template <typename T, int KM>
+template <typename T, int KM, int P>
 __global__ void __launch_bounds__(256) combine_kernel(const uint4* __restrict__ y_perm,
                                                       const float* __restrict__ prob_perm,
                                                       const int32_t* __restrict__ row_of_slot, int64_t Tn, int K,
                                                       int vpr, uint4* __restrict__ y) {
   constexpr int NV = Vec<T>::N;
   const int lane = threadIdx.x & 31;
-  const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const auto [t, part] = warp_token<P>();
   if (t >= Tn) return;
   int32_t rows[KM];
   load_rows<KM>(row_of_slot, t, K, rows);
   float p[KM];
 #pragma unroll
   for (int k = 0; k < KM; ++k) p[k] = (k < K) ? __ldg(prob_perm + rows[k]) : 0.f;
-  for (int v = lane; v < vpr; v += 32) {
+  for (int v = part * 32 + lane; v < vpr; v += 32 * P) {
     uint4 raw[KM];
 #pragma unroll
     for (int k = 0; k < KM; ++k)
@@ -256,20 +282,21 @@ cudaError_t launch_combine(const Ctx& c, DType dt, const void* y_perm, const flo
   if (T == 0) return cudaSuccess;
   const int warps = 8;
   const int vpr = (int)((int64_t)D * dsize(dt) / 16);
-  const unsigned grid = (unsigned)((T + warps - 1) / warps);
+  const int parts = row_parts(c, T, K, vpr);
+  const unsigned grid = row_grid(T, parts);
   KernelScope ks("combine", c.stream);
   if (dt == DType::BF16) {
-    MOE_DISPATCH_KM(K, (combine_kernel<bf16, KM><<<grid, 32 * warps, 0, c.stream>>>(
+    MOE_DISPATCH_KM_P(K, parts, (combine_kernel<bf16, KM, P><<<grid, 32 * warps, 0, c.stream>>>(
                            (const uint4*)y_perm, prob_perm, row_of_slot, T, K, vpr, (uint4*)y)));
   } else {
-    MOE_DISPATCH_KM(K, (combine_kernel<float, KM><<<grid, 32 * warps, 0, c.stream>>>(
+    MOE_DISPATCH_KM_P(K, parts, (combine_kernel<float, KM, P><<<grid, 32 * warps, 0, c.stream>>>(
                            (const uint4*)y_perm, prob_perm, row_of_slot, T, K, vpr, (uint4*)y)));
   }
   return cudaGetLastError();
 }
 
 // Combine backward: dY_perm[row_k] = p_k dy[t]; dprob_perm[row_k] = <dy[t], Y_perm[row_k]>.
-template <typename T, int KM>
+template <typename T, int KM, int P>
 __global__ void __launch_bounds__(256) combine_bwd_kernel(const uint4* __restrict__ dy,
                                                           const uint4* __restrict__ y_perm,
                                                           const float* __restrict__ prob_perm,
@@ -278,46 +305,59 @@ __global__ void __launch_bounds__(256) combine_bwd_kernel(const uint4* __restric
                                                           float* __restrict__ dprob_perm) {
   constexpr int NV = Vec<T>::N;
   const int lane = threadIdx.x & 31;
-  const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (t >= Tn) return;
-  int32_t rows[KM];
-  load_rows<KM>(row_of_slot, t, K, rows);
-  float p[KM], dot[KM];
+  __shared__ float s_dot[8][KM];  // a warp's share of each dot product (P > 1)
+  const auto [t, part] = warp_token<P>();
+  const int warp = threadIdx.x >> 5;
+  if (t < Tn) {
+    int32_t rows[KM];
+    load_rows<KM>(row_of_slot, t, K, rows);
+    float p[KM], dot[KM];
 #pragma unroll
-  for (int k = 0; k < KM; ++k) {
-    p[k] = (k < K) ? __ldg(prob_perm + rows[k]) : 0.f;
-    dot[k] = 0.f;
-  }
-  for (int v = lane; v < vpr; v += 32) {
-    const uint4 gv = ld_stream(dy + t * vpr + v);
-    uint4 raw[KM];
+    for (int k = 0; k < KM; ++k) {
+      p[k] = (k < K) ? __ldg(prob_perm + rows[k]) : 0.f;
+      dot[k] = 0.f;
+    }
+    for (int v = part * 32 + lane; v < vpr; v += 32 * P) {
+      const uint4 gv = ld_stream(dy + t * vpr + v);
+      uint4 raw[KM];
 #pragma unroll
-    for (int k = 0; k < KM; ++k)
-      if (k < K) raw[k] = ld_stream(y_perm + (int64_t)rows[k] * vpr + v);
-    float g[NV];
-    unpack16<T>(gv, g);
+      for (int k = 0; k < KM; ++k)
+        if (k < K) raw[k] = ld_stream(y_perm + (int64_t)rows[k] * vpr + v);
+      float g[NV];
+      unpack16<T>(gv, g);
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        if (k < K) {
+          float f[NV], o[NV];
+          unpack16<T>(raw[k], f);
+#pragma unroll
+          for (int i = 0; i < NV; ++i) {
+            dot[k] = fmaf(g[i], f[i], dot[k]);
+            o[i] = p[k] * g[i];
+          }
+          st_stream(dy_perm + (int64_t)rows[k] * vpr + v, pack16<T>(o));
+        }
+      }
+    }
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
       if (k < K) {
-        float f[NV], o[NV];
-        unpack16<T>(raw[k], f);
+        float s = dot[k];
 #pragma unroll
-        for (int i = 0; i < NV; ++i) {
-          dot[k] = fmaf(g[i], f[i], dot[k]);
-          o[i] = p[k] * g[i];
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) {
+          if (P == 1) dprob_perm[rows[k]] = s;
+          else s_dot[warp][k] = s;
         }
-        st_stream(dy_perm + (int64_t)rows[k] * vpr + v, pack16<T>(o));
       }
     }
   }
-#pragma unroll
-  for (int k = 0; k < KM; ++k) {
-    if (k < K) {
-      float s = dot[k];
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-      if (lane == 0) dprob_perm[rows[k]] = s;
-    }
+  if (P == 1) return;  // the same for the whole grid
+  __syncthreads();
+  if (t < Tn && part == 0 && lane < K) {
+    float s = 0.f;
+    for (int j = 0; j < P; ++j) s += s_dot[warp + j][lane];
+    dprob_perm[__ldg(row_of_slot + t * K + lane)] = s;
   }
 }
 
@@ -327,14 +367,15 @@ cudaError_t launch_combine_bwd(const Ctx& c, DType dt, const void* dy, const voi
   if (T == 0) return cudaSuccess;
   const int warps = 8;
   const int vpr = (int)((int64_t)D * dsize(dt) / 16);
-  const unsigned grid = (unsigned)((T + warps - 1) / warps);
+  const int parts = row_parts(c, T, K, vpr);
+  const unsigned grid = row_grid(T, parts);
   KernelScope ks("combine_bwd", c.stream);
   if (dt == DType::BF16) {
-    MOE_DISPATCH_KM(K, (combine_bwd_kernel<bf16, KM><<<grid, 32 * warps, 0, c.stream>>>(
+    MOE_DISPATCH_KM_P(K, parts, (combine_bwd_kernel<bf16, KM, P><<<grid, 32 * warps, 0, c.stream>>>(
                            (const uint4*)dy, (const uint4*)y_perm, prob_perm, row_of_slot, T, K, vpr,
                            (uint4*)dy_perm, dprob_perm)));
   } else {
-    MOE_DISPATCH_KM(K, (combine_bwd_kernel<float, KM><<<grid, 32 * warps, 0, c.stream>>>(
+    MOE_DISPATCH_KM_P(K, parts, (combine_bwd_kernel<float, KM, P><<<grid, 32 * warps, 0, c.stream>>>(
                            (const uint4*)dy, (const uint4*)y_perm, prob_perm, row_of_slot, T, K, vpr,
                            (uint4*)dy_perm, dprob_perm)));
   }
@@ -343,7 +384,7 @@ cudaError_t launch_combine_bwd(const Ctx& c, DType dt, const void* dy, const voi
 
 // Dispatch backward: dx[t] = sum_k dX_perm[row_k] (fp32 accumulation; dx
 // rows ldv 16-byte vectors apart); dprob[t, k] = dprob_perm[row_k].
-template <typename T, int KM>
+template <typename T, int KM, int P>
 __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const uint4* __restrict__ dx_perm,
                                                            const float* __restrict__ dprob_perm,
                                                            const int32_t* __restrict__ row_of_slot, int64_t Tn,
@@ -351,11 +392,11 @@ __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const uint4* __restri
                                                            float* __restrict__ dprob) {
   constexpr int NV = Vec<T>::N;
   const int lane = threadIdx.x & 31;
-  const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const auto [t, part] = warp_token<P>();
   if (t >= Tn) return;
   int32_t rows[KM];
   load_rows<KM>(row_of_slot, t, K, rows);
-  for (int v = lane; v < vpr; v += 32) {
+  for (int v = part * 32 + lane; v < vpr; v += 32 * P) {
     uint4 raw[KM];
 #pragma unroll
     for (int k = 0; k < KM; ++k)
@@ -375,7 +416,7 @@ __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const uint4* __restri
     st_stream(dx + t * ldv + v, pack16<T>(acc));
   }
   // the probability gradients last, off the path of the row loads
-  if (lane < K) dprob[t * K + lane] = __ldg(dprob_perm + row_of_slot[t * K + lane]);
+  if (part == 0 && lane < K) dprob[t * K + lane] = __ldg(dprob_perm + row_of_slot[t * K + lane]);
 }
 
 cudaError_t launch_dispatch_bwd(const Ctx& c, DType dt, const void* dx_perm, const float* dprob_perm,
@@ -384,14 +425,15 @@ cudaError_t launch_dispatch_bwd(const Ctx& c, DType dt, const void* dx_perm, con
   if (T == 0) return cudaSuccess;
   const int warps = 8;
   const int vpr = (int)((int64_t)D * dsize(dt) / 16);
+  const int parts = row_parts(c, T, K, vpr);
+  const unsigned grid = row_grid(T, parts);
   const int64_t ldv = (ldx > 0 ? ldx : D) * (int64_t)dsize(dt) / 16;
-  const unsigned grid = (unsigned)((T + warps - 1) / warps);
   KernelScope ks("dispatch_bwd", c.stream);
   if (dt == DType::BF16) {
-    MOE_DISPATCH_KM(K, (dispatch_bwd_kernel<bf16, KM><<<grid, 32 * warps, 0, c.stream>>>(
+    MOE_DISPATCH_KM_P(K, parts, (dispatch_bwd_kernel<bf16, KM, P><<<grid, 32 * warps, 0, c.stream>>>(
                            (const uint4*)dx_perm, dprob_perm, row_of_slot, T, K, vpr, ldv, (uint4*)dx, dprob)));
   } else {
-    MOE_DISPATCH_KM(K, (dispatch_bwd_kernel<float, KM><<<grid, 32 * warps, 0, c.stream>>>(
+    MOE_DISPATCH_KM_P(K, parts, (dispatch_bwd_kernel<float, KM, P><<<grid, 32 * warps, 0, c.stream>>>(
                            (const uint4*)dx_perm, dprob_perm, row_of_slot, T, K, vpr, ldv, (uint4*)dx, dprob)));
   }
   return cudaGetLastError();
@@ -408,7 +450,7 @@ cudaError_t launch_dispatch_bwd(const Ctx& c, DType dt, const void* dx_perm, con
 //   dx[t]       = sum_k dX_perm[row_k] + sum_k dz[t, e_k] W_r[e_k]
 //                 (fp32 accumulation, rounded once).
 // dz16 (bf16 copy of dz, for the router weight gradient) may be NULL.
-template <typename T, int KM>
+template <typename T, int KM, int P>
 __global__ void __launch_bounds__(256, KM <= 8 ? 3 : 1) dispatch_route_bwd_kernel(
     const uint4* __restrict__ dx_perm, const float* __restrict__ dprob_perm, const int32_t* __restrict__ row_of_slot,
     const int32_t* __restrict__ idx, const float* __restrict__ prob, const uint4* __restrict__ w_router, int64_t Tn,
@@ -416,7 +458,7 @@ __global__ void __launch_bounds__(256, KM <= 8 ? 3 : 1) dispatch_route_bwd_kerne
     bf16* __restrict__ dz16, uint32_t* err) {
   constexpr int NV = Vec<T>::N;
   const int lane = threadIdx.x & 31;
-  const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const auto [t, part] = warp_token<P>();
   if (t >= Tn) return;
   int32_t rows[KM];
   load_rows<KM>(row_of_slot, t, K, rows);
@@ -442,7 +484,7 @@ __global__ void __launch_bounds__(256, KM <= 8 ? 3 : 1) dispatch_route_bwd_kerne
       ek[k] = -1;
     }
   }
-  for (int v = lane; v < vpr; v += 32) {
+  for (int v = part * 32 + lane; v < vpr; v += 32 * P) {
     // the K dX_perm rows (HBM) first, then the K rows of W_r (L2-resident):
     // one set of K vectors in registers at a time keeps three blocks per SM
     uint4 raw[KM];
@@ -475,8 +517,8 @@ __global__ void __launch_bounds__(256, KM <= 8 ? 3 : 1) dispatch_route_bwd_kerne
     }
     st_stream(dx + t * vpr + v, pack16<T>(acc));
   }
-  if (lane < K) dprob[t * K + lane] = my_dp;
-  for (int e0 = 0; e0 < E; e0 += 32) {
+  if (part == 0 && lane < K) dprob[t * K + lane] = my_dp;
+  for (int e0 = part * 32; e0 < E; e0 += 32 * P) {
     const int e = e0 + lane;
     float val = 0.f;
 #pragma unroll
@@ -496,14 +538,15 @@ cudaError_t launch_dispatch_route_bwd(const Ctx& c, DType dt, const void* dx_per
   if (T == 0) return cudaSuccess;
   const int warps = 8;
   const int vpr = (int)((int64_t)D * dsize(dt) / 16);
-  const unsigned grid = (unsigned)((T + warps - 1) / warps);
+  const int parts = row_parts(c, T, K, vpr);
+  const unsigned grid = row_grid(T, parts);
   KernelScope ks("dispatch_route_bwd", c.stream);
   if (dt == DType::BF16) {
-    MOE_DISPATCH_KM(K, (dispatch_route_bwd_kernel<bf16, KM><<<grid, 32 * warps, 0, c.stream>>>(
+    MOE_DISPATCH_KM_P(K, parts, (dispatch_route_bwd_kernel<bf16, KM, P><<<grid, 32 * warps, 0, c.stream>>>(
                            (const uint4*)dx_perm, dprob_perm, row_of_slot, idx, prob, (const uint4*)w_router, T, K,
                            E, vpr, (uint4*)dx, dprob, dz, (bf16*)dz16, c.err)));
   } else {
-    MOE_DISPATCH_KM(K, (dispatch_route_bwd_kernel<float, KM><<<grid, 32 * warps, 0, c.stream>>>(
+    MOE_DISPATCH_KM_P(K, parts, (dispatch_route_bwd_kernel<float, KM, P><<<grid, 32 * warps, 0, c.stream>>>(
                            (const uint4*)dx_perm, dprob_perm, row_of_slot, idx, prob, (const uint4*)w_router, T, K,
                            E, vpr, (uint4*)dx, dprob, dz, (bf16*)dz16, c.err)));
   }
