@@ -19,9 +19,9 @@ size_t perm_workspace_bytes(int64_t TK, int E) {
 }
 
 // Per-chunk expert histogram (shared-memory counters; counts are order-free,
-// so the result is deterministic).  Layout: counts[e * nchunks + chunk].
+// so the result is deterministic).  Layout: counts[chunk * E + e].
 __global__ void __launch_bounds__(256) perm_hist_kernel(const int32_t* __restrict__ idx, int64_t TK, int E,
-                                                        int nchunks, int32_t* __restrict__ counts, uint32_t* err) {
+                                                        int32_t* __restrict__ counts, uint32_t* err) {
   __shared__ int h[kMaxE];
   for (int i = threadIdx.x; i < E; i += blockDim.x) h[i] = 0;
   __syncthreads();
@@ -42,54 +42,30 @@ __global__ void __launch_bounds__(256) perm_hist_kernel(const int32_t* __restric
     else set_error(err, kErrIndex);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < E; i += blockDim.x) counts[(int64_t)i * nchunks + blockIdx.x] = h[i];
+  for (int i = threadIdx.x; i < E; i += blockDim.x) counts[(int64_t)blockIdx.x * E + i] = h[i];
 }
 
 // Ranks every slot of one chunk in slot order (= token order within an
 // expert, since a token picks an expert at most once), so the permutation is
 // stable in t and bit-reproducible.  Each block first derives its chunk's
-// first row per expert from the whole (expert, chunk) count table: the
+// first row per expert from the whole (chunk, expert) count table: the
 // exclusive scan of the experts' totals plus the expert's counts in the
-// earlier chunks (block 0 also writes the offsets).  Warp w owns slots
+// earlier chunks (block 0 also writes the offsets); a single chunk (nchunks 1)
+// counts its own slots and needs no table.  Warp w owns slots
 // [w * kSub, (w+1) * kSub) of the chunk and walks them 32 at a time; lanes
 // that share an expert get consecutive rows by __match_any_sync rank.  Also
-// writes prob_perm.
+// writes prob_perm.  Bound by its chain of round trips: 16 of a table column's
+// counts are in flight at once, and one thread per expert scans the totals by
+// shuffles: 64 chunks of E = 256 16.9 -> 10.6 us.
 __global__ void __launch_bounds__(kRankWarps * 32) perm_rank_kernel(
     const int32_t* __restrict__ idx, const float* __restrict__ prob, int64_t TK, int K, int E, int nchunks,
     const int32_t* __restrict__ counts, int32_t* __restrict__ offsets, int32_t* __restrict__ row_of_slot,
-    int32_t* __restrict__ token_of_row, float* __restrict__ prob_perm) {
+    int32_t* __restrict__ token_of_row, float* __restrict__ prob_perm, uint32_t* err) {
+  static_assert(kRankWarps * 32 >= kMaxE, "one thread per expert");
   __shared__ int cnt[kRankWarps * kMaxE];
-  __shared__ int tot[kMaxE + 1];  // expert totals, then their exclusive scan
-  __shared__ int pre[kMaxE];      // the expert's slots in the chunks before this one
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < kRankWarps * E; i += blockDim.x) cnt[i] = 0;
-  for (int e = threadIdx.x; e < E; e += blockDim.x) {
-    const int32_t* row = counts + (int64_t)e * nchunks;
-    int before = 0, all = 0;
-#pragma unroll 8
-    for (int c = 0; c < nchunks; ++c) {
-      const int v = row[c];
-      before += c < (int)blockIdx.x ? v : 0;
-      all += v;
-    }
-    pre[e] = before;
-    tot[e] = all;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {  // E <= 256: a serial scan is a few hundred adds
-    int run = 0;
-    for (int e = 0; e < E; ++e) {
-      const int v = tot[e];
-      tot[e] = run;
-      run += v;
-    }
-    tot[E] = run;
-  }
-  __syncthreads();
-  if (blockIdx.x == 0)
-    for (int e = threadIdx.x; e <= E; e += blockDim.x) offsets[e] = tot[e];
-  const int64_t c0 = (int64_t)blockIdx.x * kChunk;
-  const int64_t w0 = c0 + (int64_t)warp * kSub;
+  __shared__ int wsum[kRankWarps];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t w0 = (int64_t)blockIdx.x * kChunk + (int64_t)warp * kSub;
   const int64_t w1 = min(TK, w0 + kSub);
   // the warp's kSub expert indices and probabilities, all loads in flight at
   // once (expert -1 past the end)
@@ -101,15 +77,48 @@ __global__ void __launch_bounds__(kRankWarps * 32) perm_rank_kernel(
     ev[i] = s < w1 ? __ldg(idx + s) : -1;
     pv[i] = s < w1 ? __ldg(prob + s) : 0.f;
   }
+  for (int i = tid; i < kRankWarps * E; i += kRankWarps * 32) cnt[i] = 0;
+  int before = 0, all = 0;  // expert tid's slots in the chunks before this one, and in all
+  if (nchunks > 1 && tid < E) {
+    constexpr int U = 16;
+    for (int c0 = 0; c0 < nchunks; c0 += U) {
+      int v[U];
 #pragma unroll
-  for (int i = 0; i < kSub / 32; ++i)
-    if (ev[i] >= 0 && ev[i] < E) atomicAdd(&cnt[warp * E + ev[i]], 1);
+      for (int u = 0; u < U; ++u) v[u] = c0 + u < nchunks ? __ldg(counts + (int64_t)(c0 + u) * E + tid) : 0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        before += c0 + u < (int)blockIdx.x ? v[u] : 0;
+        all += v[u];
+      }
+    }
+  }
   __syncthreads();
-  for (int e = threadIdx.x; e < E; e += blockDim.x) {
-    int run = tot[e] + pre[e];
+#pragma unroll
+  for (int i = 0; i < kSub / 32; ++i) {
+    if (ev[i] >= 0 && ev[i] < E) atomicAdd(&cnt[warp * E + ev[i]], 1);
+    else if (nchunks == 1 && w0 + i * 32 + lane < w1) set_error(err, kErrIndex);  // (the histogram did otherwise)
+  }
+  __syncthreads();
+  if (nchunks == 1 && tid < E)
+    for (int w = 0; w < kRankWarps; ++w) all += cnt[w * E + tid];
+  int inc = all;  // inclusive scan over the experts
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) wsum[warp] = inc;
+  __syncthreads();
+  for (int w = 0; w < warp; ++w) inc += wsum[w];
+  if (tid < E) {
+    if (blockIdx.x == 0) {
+      offsets[tid] = inc - all;
+      if (tid == E - 1) offsets[E] = inc;
+    }
+    int run = inc - all + before;
     for (int w = 0; w < kRankWarps; ++w) {
-      const int c = cnt[w * E + e];
-      cnt[w * E + e] = run;
+      const int c = cnt[w * E + tid];
+      cnt[w * E + tid] = run;
       run += c;
     }
   }
@@ -147,16 +156,16 @@ cudaError_t launch_permutation(const Ctx& c, const int32_t* idx, const float* pr
     KernelScope ks("perm_zero", c.stream);
     return cudaMemsetAsync(offsets, 0, sizeof(int32_t) * (E + 1), c.stream);
   }
-  {
+  if (nch > 1) {
     KernelScope ks("perm_hist", c.stream);
-    perm_hist_kernel<<<nch, 256, 0, c.stream>>>(idx, TK, E, nch, counts, c.err);
+    perm_hist_kernel<<<nch, 256, 0, c.stream>>>(idx, TK, E, counts, c.err);
+    cudaError_t st = cudaGetLastError();
+    if (st != cudaSuccess) return st;
   }
-  cudaError_t st = cudaGetLastError();
-  if (st != cudaSuccess) return st;
   {
     KernelScope ks("perm_rank", c.stream);
     perm_rank_kernel<<<nch, kRankWarps * 32, 0, c.stream>>>(idx, prob, TK, K, E, nch, counts, offsets,
-                                                            row_of_slot, token_of_row, prob_perm);
+                                                            row_of_slot, token_of_row, prob_perm, c.err);
   }
   return cudaGetLastError();
 }
