@@ -196,13 +196,17 @@ int router_splits(const Dims& d, int num_sms) {
   return s < 1 ? 1 : (int)s;
 }
 // The same for the CUDA-core engine (fp32 inputs, or a number of experts that
-// the tensor-core engine does not take), which covers a thin output with 32 x 32
-// tiles: the three blocks per SM that fit, each reducing at least 256 tokens.
+// the tensor-core engine does not take).  Up to 32 experts: 32 x 32 tiles, the
+// three blocks per SM that fit, each reducing at least 256 tokens.  More: enough
+// splits for two 64 x 128 tiles per SM, which do twice the products per staged
+// element, down to 128 tokens: bf16 T = 2045, E = 60, Din = 2048 41 us on 32 x 32
+// tiles, 23 now.
 int router_splits_simt(const Dims& d, int num_sms) {
-  const int64_t tiles = (int64_t)((d.E + 31) / 32) * ((d.Din + 31) / 32);
-  int64_t s = 3 * num_sms / tiles;
+  const bool thin = d.E <= 32;
+  const int64_t tiles = thin ? (d.Din + 31) / 32 : (int64_t)((d.E + 63) / 64) * ((d.Din + 127) / 128);
+  int64_t s = (thin ? 3 : 2) * num_sms / tiles;
   if (s > kRouterSplits) s = kRouterSplits;
-  if (s > d.T / 256) s = d.T / 256;
+  if (s > d.T / (thin ? 256 : 128)) s = d.T / (thin ? 256 : 128);
   return s < 1 ? 1 : (int)s;
 }
 // Sigmoid router forward: per-token score sums and the balance statistics'
@@ -891,7 +895,7 @@ static int router_grad_gemms(const Ctx& c, const Dims& d, const void* x, const v
   if (simt_splits > 1) {
     // the same split for the CUDA-core engine: without it the few tiles of an
     // E x Din output each walk all T tokens (fp32 T = 3001, E = 12, Din = 512:
-    // 627 us; bf16 T = 2045, E = 60, Din = 2048: 451 us; now 17 and 44 us)
+    // 627 us; bf16 T = 2045, E = 60, Din = 2048: 451 us; now 17 and 23 us)
     GemmDesc bs = b;
     bs.group = Group::K;
     bs.num_groups = simt_splits;
