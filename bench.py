@@ -81,7 +81,6 @@ def kernel_work(name: str, w: synth.Workload, T: int, Fs: int = 0, latent_fused:
         "select_sigmoid": T * E * 4 + T * K * 8,
         "balance_finalize": 0.0,
         "route_dz_sigmoid": T * E * 4 + T * K * 12 + T * E * 6,
-        "swiglu_bwd": 5.0 * TK * F * bx,
         "relusq_bwd": 3.0 * T * Fs * bx,
         "dispatch_fp8": T * D * bx + TK * D + 8 * TK,
         "dequant_rows": TK * D + TK * D * bx + 4 * TK,
@@ -622,7 +621,7 @@ def main() -> None:
     kernels = kernel_table(r["prof"], args.steps, w, T, args.shared_width, r["latent_fused"], peaks)
     roof = top_roofline(kernels, w, peaks)
 
-    exp_ms = sum(v["ms_per_step"] for k, v in kernels.items() if k.startswith("ffn") or k == "swiglu_bwd")
+    exp_ms = sum(v["ms_per_step"] for k, v in kernels.items() if k.startswith("ffn"))
     perm_names = ("dispatch_rows", "combine", "combine_bwd", "dispatch_bwd", "dispatch_route_bwd")
     perm_ms = sum(v["ms_per_step"] for k, v in kernels.items() if k in perm_names)
 

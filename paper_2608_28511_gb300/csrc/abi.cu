@@ -172,9 +172,9 @@ size_t align_up(size_t v) { return (v + 255) & ~size_t(255); }
 // Workspace carve-up.  Calls are ordered on one stream, so the regions used by
 // different calls may overlap.
 size_t ws_perm(const Dims& d) { return align_up(perm_workspace_bytes(d.TK, d.E)); }
-// dH [TK, 2F], dA [TK, F], then the two wgrad GEMMs' per-expert tail tensor
-// maps (one region each: one launch builds both)
-size_t ws_ffn_bwd_maps_offset(const Dims& d) { return align_up((size_t)d.TK * 3 * d.F * d.bx); }
+// dH [TK, 2F], then the two wgrad GEMMs' per-expert tail tensor maps (one
+// region each: one launch builds both)
+size_t ws_ffn_bwd_maps_offset(const Dims& d) { return align_up((size_t)d.TK * 2 * d.F * d.bx); }
 size_t ws_ffn_bwd_maps_bytes(const Dims& d) { return align_up(gemm_tc_group_scratch_bytes(d.E)); }
 size_t ws_ffn_bwd(const Dims& d) { return ws_ffn_bwd_maps_offset(d) + 2 * ws_ffn_bwd_maps_bytes(d); }
 // Router weight gradient: split-K over the T tokens into at most kRouterSplits
@@ -608,13 +608,14 @@ static int expert_ffn_bwd_impl(const Ctx& c, const Dims& d, const void* dy_perm,
                                const int32_t* expert_offsets, const void* w1, const void* w2, void* dx_perm,
                                float* dw1, float* dw2, void* ws) {
   void* dH = ws;
-  void* dA = static_cast<char*>(ws) + (size_t)d.TK * 2 * d.F * d.bx;
   void* maps = static_cast<char*>(ws) + ws_ffn_bwd_maps_offset(d);
   void* maps1 = static_cast<char*>(maps) + ws_ffn_bwd_maps_bytes(d);
-  // dgrad-2: dA = dy_perm . w2_e, then the SwiGLU backward dA, h -> dH
+  // dgrad-2: dA = dy_perm . w2_e, with the SwiGLU backward dA, h -> dH in its
+  // epilogue (dA itself is never stored)
   GemmDesc a;
   a.group = Group::M;
-  a.epi = Epi::Store;
+  a.epi = Epi::SwigluBwd;
+  a.aux = const_cast<void*>(h_save);
   a.N = d.F;
   a.K = d.D;
   a.num_groups = d.E;
@@ -629,9 +630,9 @@ static int expert_ffn_bwd_impl(const Ctx& c, const Dims& d, const void* dy_perm,
   a.sb_n = 1;
   a.sb_k = d.F;
   a.sb_g = (int64_t)d.D * d.F;
-  a.C = dA;
+  a.C = dH;
   a.c_type = d.dt;
-  a.ldc = d.F;
+  a.ldc = 2 * d.F;
   // wgrad-2: dw2_e[d, f] = sum_rows dy_perm[r, d] a[r, f]
   GemmDesc b;
   b.group = Group::K;
@@ -699,20 +700,15 @@ static int expert_ffn_bwd_impl(const Ctx& c, const Dims& d, const void* dy_perm,
   w.c_type = DType::F32;
   w.ldc = d.D;
   w.sc_g = (int64_t)2 * d.F * d.D;
-  if (d.TK > 0) {
-    // on the tensor-core engine the SwiGLU backward runs in dgrad-2's epilogue
-    // (dA stays in TMEM: h in, dH out); otherwise as a separate pass over dA
-    GemmDesc af = a;
-    af.epi = Epi::SwigluBwd;
-    af.aux = const_cast<void*>(h_save);
-    af.C = dH;
-    af.ldc = 2 * d.F;
-    if (gemm_tc_supports(af)) {
-      TRY_CUDA(launch_gemm_tc(c, af, "ffn2_dgrad_swiglu_tc"));
-    } else {
-      TRY_CUDA(gemm(c, a, "ffn2_dgrad_tc", "ffn2_dgrad_simt"));
-      TRY_CUDA(launch_swiglu_bwd(c, d.dt, dA, h_save, d.TK, d.F, dH));
-    }
+  if (d.TK > 0) TRY_CUDA(gemm(c, a, "ffn2_dgrad_swiglu_tc", "ffn2_dgrad_swiglu_simt"));
+  if (d.dt == DType::F32) {
+    // the three products that depend on dH, in one launch: each alone leaves SMs
+    // idle on a small batch, and in its last wave on a larger one (T = 256,
+    // D = 128, E = 8, K = 2, F = 256: 33 -> 18.5 us; T = 3001, D = 512, E = 12,
+    // K = 3, F = 768: 770 -> 712)
+    const GemmDesc all[3] = {cg, w, b};
+    TRY_CUDA(launch_gemm_simt_f32x3(c, all, "ffn_bwd_simt"));
+    return MOE_OK;
   }
   // both weight gradients' tail maps in one launch (each GEMM builds its own
   // if they are not both on the tensor-core engine)

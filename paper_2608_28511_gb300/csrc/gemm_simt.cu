@@ -13,14 +13,17 @@
 // the next k-tile's global loads are issued before the current one is
 // multiplied and written to the other buffer after it, one barrier per k-tile.
 // The products are packed fp32 FMAs on two adjacent columns (fma.rn.f32x2, each
-// half rounded as a scalar FMA), in the order of k.
+// half rounded as a scalar FMA), in the order of k.  The SwiGLU backward is an
+// epilogue of dA's product: 174 us at T = 3001 for 160 and 18.6 as a pass of its
+// own.
 //
 // Bound by the FMA pipe and its issue slots.  Measured on an fp32 layer of
 // T = 3001, D = 512, E = 12, K = 3, F = 768: GEMM-1 (14.2 GFLOP) 526 us on the
 // single-buffered 64 x 128 x 16 tiles used before, 358 us with scalar FMAs here,
-// 320 us with packed ones (44 TFLOP/s; the FMA pipe 66 % busy, 92 % of the tile
-// rows real).  A k-tile of 8 (363 us) or 32 (336 us, spills), and one block per
-// SM with more registers (365 us), are slower.
+// 304 us with packed ones (47 TFLOP/s; 92 % of the tile rows real).  A k-tile of
+// 8 (363 us) or 32 (336 us, spills), one block per SM with more registers
+// (365 us), and in the 32 x 32 tile k split over four groups of threads, are
+// slower.
 #include "common.cuh"
 #include "launch.h"
 
@@ -186,8 +189,24 @@ __device__ __forceinline__ void frag(const float* row, int t, int sw, float (&f)
   }
 }
 
-template <typename TA, typename TB, typename TC, int BM, int BN, int BK>
-__global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) simt_gemm_kernel(GemmDesc d) {
+// The problems of one launch: problem i's blocks start at first[i], tiles[i] of
+// them per group of a Group::K problem.
+template <int NP>
+struct Problems {
+  GemmDesc d[NP];
+  unsigned first[NP];
+  unsigned tiles[NP];
+};
+
+template <typename TA, typename TB, typename TC, int BM, int BN, int BK, int NP>
+__global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3)
+    simt_gemm_kernel(const __grid_constant__ Problems<NP> ps) {
+  int pi = 0;
+#pragma unroll
+  for (int i = 1; i < NP; ++i)
+    if (blockIdx.x >= ps.first[i]) pi = i;
+  const GemmDesc& d = ps.d[pi];
+  const unsigned block = blockIdx.x - ps.first[pi];
   constexpr int TM = BM / 16, TN = BN / 16;
   extern __shared__ __align__(16) float smem[];  // two A tiles, then two B tiles
   auto As = [&](int b) { return smem + b * BK * BM; };
@@ -197,9 +216,10 @@ __global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) simt_gemm_kernel
   __shared__ int s_row0, s_rend;
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
-  const int tiles_n = (int)((d.N + BN - 1) / BN);
-  const int mt = (int)(blockIdx.x / (unsigned)tiles_n);  // a row tile's column tiles are consecutive blocks
-  const int64_t n0 = (int64_t)(blockIdx.x % (unsigned)tiles_n) * BN;
+  const unsigned tiles_n = (unsigned)((d.N + BN - 1) / BN);
+  const unsigned tile = d.group == Group::K ? block % ps.tiles[pi] : block;
+  const int mt = (int)(tile / tiles_n);  // a row tile's column tiles are consecutive blocks
+  const int64_t n0 = (int64_t)(tile % tiles_n) * BN;
 
   int g = 0;
   int64_t row0 = (int64_t)mt * BM, row_end = d.M, kbeg = 0, kend = d.K;
@@ -236,7 +256,7 @@ __global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) simt_gemm_kernel
     row0 = s_row0;
     row_end = s_rend;
   } else if (d.group == Group::K) {
-    g = blockIdx.y;
+    g = (int)(block / ps.tiles[pi]);
     if (d.offsets) {
       kbeg = d.offsets[g];
       kend = d.offsets[g + 1];
@@ -326,6 +346,31 @@ __global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) simt_gemm_kernel
         if (d.epi == Epi::StoreBias && d.bias && gn + u < d.N) v[u] += d.bias[gn + u];
         if (d.epi == Epi::Accum && gn + u < d.N) v[u] = to_f32<TC>(crow[gn + u]) + v[u];
       }
+      if (d.epi == Epi::SwigluBwd) {
+        // dA at columns gn ..: the gate block of h / dH at 128 (gn / 64) + gn mod 64,
+        // the up block 64 further (N is a multiple of 64)
+        const int64_t o = gm * d.ldc + (gn >> 6) * 128 + (gn & 63);
+        const TC* h = static_cast<const TC*>(d.aux) + o;
+        float dg[CG], du[CG];
+#pragma unroll
+        for (int u = 0; u < CG; ++u) {
+          const float gate = to_f32<TC>(__ldg(h + u)), up = to_f32<TC>(__ldg(h + 64 + u));
+          const float sg = __frcp_rn(1.0f + __expf(-gate));
+          dg[u] = v[u] * up * sg * (1.0f + gate * (1.0f - sg));
+          du[u] = v[u] * gate * sg;
+        }
+        if constexpr (CG == 4) {
+          st4(C + o, dg);
+          st4(C + o + 64, du);
+        } else {
+#pragma unroll
+          for (int u = 0; u < CG; ++u) {
+            C[o + u] = from_f32<TC>(dg[u]);
+            C[o + 64 + u] = from_f32<TC>(du[u]);
+          }
+        }
+        continue;
+      }
       if (whole) {
         if constexpr (CG == 4) st4(crow + gn, v);
       } else {
@@ -353,50 +398,68 @@ __global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) simt_gemm_kernel
   }
 }
 
-template <typename TA, typename TB, typename TC, int BM, int BN, int BK>
-cudaError_t run_tile(const Ctx& c, const GemmDesc& d) {
-  const int64_t tiles_n = (d.N + BN - 1) / BN;
-  const int64_t tiles_m =
-      d.group == Group::M ? (d.max_rows + BM - 1) / BM + d.num_groups : (d.M + BM - 1) / BM;
-  const int64_t tiles = tiles_m * tiles_n;
-  const int groups = d.group == Group::K ? d.num_groups : 1;
-  if (tiles <= 0 || groups <= 0) return cudaSuccess;
-  if (tiles > 0x7fffffff) return cudaErrorInvalidConfiguration;
-  const dim3 grid((unsigned)tiles, (unsigned)groups, 1);
+template <typename TA, typename TB, typename TC, int BM, int BN, int BK, int NP>
+cudaError_t run_tile(const Ctx& c, const GemmDesc (&ds)[NP]) {
+  Problems<NP> ps;
+  int64_t blocks = 0;
+  for (int i = 0; i < NP; ++i) {
+    const GemmDesc& d = ds[i];
+    const int64_t tiles_n = (d.N + BN - 1) / BN;
+    const int64_t tiles_m =
+        d.group == Group::M ? (d.max_rows + BM - 1) / BM + d.num_groups : (d.M + BM - 1) / BM;
+    const int64_t tiles = tiles_m * tiles_n;
+    const int groups = d.group == Group::K ? d.num_groups : 1;
+    if (tiles <= 0 || groups <= 0) return NP == 1 ? cudaSuccess : cudaErrorInvalidValue;
+    ps.d[i] = d;
+    ps.first[i] = (unsigned)blocks;
+    ps.tiles[i] = (unsigned)tiles;
+    blocks += tiles * groups;
+    if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
+  }
   constexpr int kSmem = 2 * (BM + BN) * BK * 4;
   static_assert(kSmem <= 48 * 1024, "fits without opting in to more shared memory");
-  simt_gemm_kernel<TA, TB, TC, BM, BN, BK><<<grid, 256, kSmem, c.stream>>>(d);
+  simt_gemm_kernel<TA, TB, TC, BM, BN, BK, NP><<<(unsigned)blocks, 256, kSmem, c.stream>>>(ps);
   return cudaGetLastError();
 }
 
 // Tiles of a BM x BN tiling that hold rows (an upper estimate for Group::M,
 // whose experts' row counts only the device knows).
-int64_t tiles_of(const GemmDesc& d, int bm, int bn) {
-  const int64_t nt = (d.N + bn - 1) / bn;
-  if (d.group == Group::M) {
-    const int64_t groups = d.max_rows < d.num_groups ? d.max_rows : d.num_groups;
-    return nt * (d.max_rows / bm + (groups + 1) / 2);
+template <int NP>
+int64_t tiles_of(const GemmDesc (&ds)[NP], int bm, int bn) {
+  int64_t sum = 0;
+  for (const GemmDesc& d : ds) {
+    const int64_t nt = (d.N + bn - 1) / bn;
+    if (d.group == Group::M) {
+      const int64_t groups = d.max_rows < d.num_groups ? d.max_rows : d.num_groups;
+      sum += nt * (d.max_rows / bm + (groups + 1) / 2);
+    } else {
+      sum += nt * ((d.M + bm - 1) / bm) * (d.group == Group::K ? d.num_groups : 1);
+    }
   }
-  return nt * ((d.M + bm - 1) / bm) * (d.group == Group::K ? d.num_groups : 1);
+  return sum;
 }
 
-template <typename TA, typename TB, typename TC>
-cudaError_t run(const Ctx& c, const GemmDesc& d) {
-  const bool swiglu = d.epi == Epi::SwigluFwd;  // needs gate and up columns in one 128-column tile
+template <typename TA, typename TB, typename TC, int NP>
+cudaError_t run(const Ctx& c, const GemmDesc (&ds)[NP]) {
+  const bool swiglu = ds[0].epi == Epi::SwigluFwd;  // needs gate and up columns in one 128-column tile
+  int64_t widest = 0;
+  for (const GemmDesc& d : ds) widest = d.N > widest ? d.N : widest;
   if constexpr (sizeof(TA) == 4 && sizeof(TB) == 4) {
     // the largest tile that still gives every SM work: at T = 256, D = 128, E = 8,
     // K = 2, F = 256 the small tiles take GEMM-1's dgrad from 102 to 17 us
-    if (d.N > 64) {
-      if (tiles_of(d, 128, 128) >= c.num_sms) return run_tile<TA, TB, TC, 128, 128, 16>(c, d);
-      if (tiles_of(d, 64, 128) >= c.num_sms) return run_tile<TA, TB, TC, 64, 128, 16>(c, d);
-      if (swiglu) return run_tile<TA, TB, TC, 32, 128, 32>(c, d);
+    if (widest > 64) {
+      if (tiles_of(ds, 128, 128) >= c.num_sms) return run_tile<TA, TB, TC, 128, 128, 16>(c, ds);
+      if (tiles_of(ds, 64, 128) >= c.num_sms) return run_tile<TA, TB, TC, 64, 128, 16>(c, ds);
+      if (swiglu) return run_tile<TA, TB, TC, 32, 128, 32>(c, ds);
     }
-    if (tiles_of(d, 64, 64) >= c.num_sms && d.N > 32) return run_tile<TA, TB, TC, 64, 64, 32>(c, d);
-    return run_tile<TA, TB, TC, 32, 32, 32>(c, d);
+    // (three problems of unequal length: several blocks per SM, or the longest is
+    // left alone; the same case on 64 x 64 tiles 29 us, on 32 x 32 18)
+    if (tiles_of(ds, 64, 64) >= NP * c.num_sms && widest > 32) return run_tile<TA, TB, TC, 64, 64, 32>(c, ds);
+    return run_tile<TA, TB, TC, 32, 32, 32>(c, ds);
   } else {
-    if (swiglu || (d.N > 64 && tiles_of(d, 64, 128) >= c.num_sms))
-      return run_tile<TA, TB, TC, 64, 128, 16>(c, d);
-    return run_tile<TA, TB, TC, 32, 32, 32>(c, d);
+    if (swiglu || (widest > 64 && tiles_of(ds, 64, 128) >= c.num_sms))
+      return run_tile<TA, TB, TC, 64, 128, 16>(c, ds);
+    return run_tile<TA, TB, TC, 32, 32, 32>(c, ds);
   }
 }
 
@@ -404,16 +467,22 @@ cudaError_t run(const Ctx& c, const GemmDesc& d) {
 
 cudaError_t launch_gemm_simt(const Ctx& c, const GemmDesc& d, const char* name) {
   KernelScope ks(name, c.stream);
+  const GemmDesc ds[1] = {d};
   const int key = (int)d.a_type * 4 + (int)d.b_type * 2 + (int)d.c_type;
   switch (key) {
-    case 0: return run<bf16, bf16, bf16>(c, d);
-    case 1: return run<bf16, bf16, float>(c, d);
-    case 2 + 0: return run<bf16, float, bf16>(c, d);
-    case 4 + 0: return run<float, bf16, bf16>(c, d);
-    case 4 + 1: return run<float, bf16, float>(c, d);
-    case 4 + 2 + 1: return run<float, float, float>(c, d);
+    case 0: return run<bf16, bf16, bf16>(c, ds);
+    case 1: return run<bf16, bf16, float>(c, ds);
+    case 2 + 0: return run<bf16, float, bf16>(c, ds);
+    case 4 + 0: return run<float, bf16, bf16>(c, ds);
+    case 4 + 1: return run<float, bf16, float>(c, ds);
+    case 4 + 2 + 1: return run<float, float, float>(c, ds);
     default: return cudaErrorNotSupported;
   }
+}
+
+cudaError_t launch_gemm_simt_f32x3(const Ctx& c, const GemmDesc (&ds)[3], const char* name) {
+  KernelScope ks(name, c.stream);
+  return run<float, float, float>(c, ds);
 }
 
 }  // namespace moe

@@ -114,10 +114,7 @@ cudaError_t launch_dispatch_nvfp4(const Ctx& c, const void* x, const int32_t* ro
 cudaError_t launch_dequant_nvfp4(const Ctx& c, const void* xq, const uint8_t* bscale, const float* rscale,
                                  int64_t rows, int D, void* out);
 
-// swiglu.cu: dH [rows, 2F] (packed) from dA [rows, F] and the saved h [rows, 2F].
-cudaError_t launch_swiglu_bwd(const Ctx& c, DType dt, const void* dA, const void* h, int64_t rows, int F,
-                              void* dH);
-// swiglu.cu: dh = 2 max(h, 0) dA over n elements (dh may alias dA).
+// relusq.cu: dh = 2 max(h, 0) dA over n elements (dh may alias dA).
 cudaError_t launch_relusq_bwd(const Ctx& c, DType dt, const void* dA, const void* h, int64_t n, void* dh);
 
 // ---------------------------------------------------------------------------
@@ -170,6 +167,9 @@ struct GemmDesc {
 };
 
 cudaError_t launch_gemm_simt(const Ctx& c, const GemmDesc& d, const char* name);
+// Three independent fp32 products in one launch; the longest reduction comes
+// first, so that the short ones fill in behind it.
+cudaError_t launch_gemm_simt_f32x3(const Ctx& c, const GemmDesc (&ds)[3], const char* name);
 
 // tcgen05 / TMA engine (bf16 operands only).  Returns cudaErrorNotSupported
 // for a descriptor it does not handle.
