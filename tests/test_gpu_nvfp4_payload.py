@@ -171,3 +171,24 @@ def test_nvfp4_payload_rejects_fp32():
                                z(16, d=torch.int32), z(16, d=torch.int32), z(16, 32, d=torch.uint8),
                                z(16, 4, d=torch.uint8), z(16), z(16), z(1 << 16, d=torch.uint8))
     assert e.value.status == -8
+
+
+@pytest.mark.parametrize("exp", [-126, -116, -101, -100, -99, -20, 0, 60, 90, 99, 100, 101])
+def test_midpoints_of_every_block_scale(exp):
+    """Every E2M1 midpoint, its bf16 neighbours and 6 times the block scale, for
+    all eight mantissas of the E4M3 block scale at three exponents, in rows whose
+    scale g puts s_b g on both sides of the reciprocal's range."""
+    mids = torch.tensor([0.25, 0.75, 1.25, 1.75, 2.5, 3.5, 5.0])
+    blocks = [torch.full((16,), 2688.0)]  # the row maximum: g = 2^exp
+    for e in (-3, 0, 4):
+        for m in range(8, 16):
+            sb = m / 8.0 * 2.0 ** e
+            v = (mids * sb).bfloat16()
+            up = (v.view(torch.int16) + 1).view(torch.bfloat16)
+            dn = (v.view(torch.int16) - 1).view(torch.bfloat16)
+            for n in (v, up, dn):
+                blocks.append(torch.cat([n.float(), -n.float(), torch.tensor([6.0 * sb, -6.0 * sb])]))
+    while len(blocks) % 4:
+        blocks.append(torch.zeros(16))
+    x = torch.cat(blocks).double() * 2.0 ** exp
+    _check_direct(torch.stack([x, -x]).to(torch.bfloat16), K=1, E=4)
