@@ -89,8 +89,10 @@ __device__ __forceinline__ void quantize_block(const uint4& v0, const uint4& v1,
 }
 
 // One warp per token: the row maximum and scale, then every block's scale and
-// codes, written to each of the token's K rows (row_of_slot).
-template <int KM>
+// codes, written to each of the token's K rows (row_of_slot).  NB > 0: a lane's
+// (at most NB) blocks are read once, into registers; wider rows are read twice.
+// T = 8191, K = 6, D = 2048, dispatch and arrival: 69.8 -> 67.8 us.
+template <int KM, int NB>
 __global__ void __launch_bounds__(256) dispatch_nvfp4_kernel(const uint4* __restrict__ x,
                                                              const int32_t* __restrict__ row_of_slot, int64_t T,
                                                              int K, int vpr, uint2* __restrict__ xq,
@@ -102,11 +104,29 @@ __global__ void __launch_bounds__(256) dispatch_nvfp4_kernel(const uint4* __rest
   const uint4* row = x + t * vpr;
   const int nblk = vpr / 2;  // 16-element blocks per row
   float amax = 0.f;
-  for (int i = lane; i < vpr; i += 32) {
-    float f[8];
-    unpack16<bf16>(__ldg(row + i), f);
+  uint4 raw[NB > 0 ? 2 * NB : 1];
+  if (NB > 0) {
+    // the lane's NB blocks stay in registers, all loads in flight at once
 #pragma unroll
-    for (int j = 0; j < 8; ++j) amax = fmaxf(amax, fabsf(f[j]));
+    for (int j = 0; j < NB; ++j) {
+      const int b = lane + 32 * j;
+      raw[2 * j] = b < nblk ? ld_stream(row + 2 * b) : make_uint4(0, 0, 0, 0);
+      raw[2 * j + 1] = b < nblk ? ld_stream(row + 2 * b + 1) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int j = 0; j < 2 * NB; ++j) {
+      float f[8];
+      unpack16<bf16>(raw[j], f);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) amax = fmaxf(amax, fabsf(f[u]));
+    }
+  } else {
+    for (int i = lane; i < vpr; i += 32) {
+      float f[8];
+      unpack16<bf16>(__ldg(row + i), f);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) amax = fmaxf(amax, fabsf(f[j]));
+    }
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
@@ -127,10 +147,10 @@ __global__ void __launch_bounds__(256) dispatch_nvfp4_kernel(const uint4* __rest
     for (int k = 0; k < KM; ++k)
       if (k == lane && dst[k] >= 0) rscale[dst[k]] = g;
   }
-  for (int b = lane; b < nblk; b += 32) {
+  auto put = [&](int b, const uint4& v0, const uint4& v1) {
     uint8_t sc;
     uint2 q;
-    quantize_block(__ldg(row + 2 * b), __ldg(row + 2 * b + 1), six_g, g, &sc, &q);
+    quantize_block(v0, v1, six_g, g, &sc, &q);
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
       if (dst[k] >= 0) {
@@ -138,6 +158,13 @@ __global__ void __launch_bounds__(256) dispatch_nvfp4_kernel(const uint4* __rest
         bscale[dst[k] * nblk + b] = sc;
       }
     }
+  };
+  if (NB > 0) {
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+      if (lane + 32 * j < nblk) put(lane + 32 * j, raw[2 * j], raw[2 * j + 1]);
+  } else {
+    for (int b = lane; b < nblk; b += 32) put(b, __ldg(row + 2 * b), __ldg(row + 2 * b + 1));
   }
 }
 
@@ -197,15 +224,16 @@ cudaError_t launch_dispatch_nvfp4(const Ctx& c, const void* x, const int32_t* ro
   const dim3 grid((unsigned)((T + warps - 1) / warps));
   const int vpr = D / 8;
   KernelScope ks("dispatch_nvfp4", c.stream);
+  auto run = [&](auto kernel) {
+    kernel<<<grid, 32 * warps, 0, c.stream>>>((const uint4*)x, row_of_slot, T, K, vpr, (uint2*)xq, bscale, rscale,
+                                              c.err);
+  };
+  const bool regs = D <= 2048;
   switch (k_bound(K)) {
-    case 2: dispatch_nvfp4_kernel<2><<<grid, 32 * warps, 0, c.stream>>>((const uint4*)x, row_of_slot, T, K, vpr,
-                       (uint2*)xq, bscale, rscale, c.err); break;
-    case 4: dispatch_nvfp4_kernel<4><<<grid, 32 * warps, 0, c.stream>>>((const uint4*)x, row_of_slot, T, K, vpr,
-                       (uint2*)xq, bscale, rscale, c.err); break;
-    case 8: dispatch_nvfp4_kernel<8><<<grid, 32 * warps, 0, c.stream>>>((const uint4*)x, row_of_slot, T, K, vpr,
-                       (uint2*)xq, bscale, rscale, c.err); break;
-    default: dispatch_nvfp4_kernel<16><<<grid, 32 * warps, 0, c.stream>>>((const uint4*)x, row_of_slot, T, K,
-                        vpr, (uint2*)xq, bscale, rscale, c.err); break;
+    case 2: regs ? run(dispatch_nvfp4_kernel<2, 4>) : run(dispatch_nvfp4_kernel<2, 0>); break;
+    case 4: regs ? run(dispatch_nvfp4_kernel<4, 4>) : run(dispatch_nvfp4_kernel<4, 0>); break;
+    case 8: regs ? run(dispatch_nvfp4_kernel<8, 4>) : run(dispatch_nvfp4_kernel<8, 0>); break;
+    default: regs ? run(dispatch_nvfp4_kernel<16, 4>) : run(dispatch_nvfp4_kernel<16, 0>); break;
   }
   return cudaGetLastError();
 }
