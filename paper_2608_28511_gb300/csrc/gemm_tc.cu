@@ -50,6 +50,19 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// C of a Group::K GEMM as [groups][m][n] fp32, boxes of 32 x 32 of one group.
+bool make_store_map(CUtensorMap* m, const GemmDesc& d) {
+  EncodeFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)d.N, (cuuint64_t)d.M, (cuuint64_t)d.num_groups};
+  cuuint64_t strides[2] = {(cuuint64_t)d.ldc * 4, (cuuint64_t)d.sc_g * 4};
+  cuuint32_t box[3] = {32, 32, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, d.C, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool al16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 // Group::K tail templates, one per row count r = 1 .. BK - 1, for MN-major A
@@ -326,10 +339,19 @@ cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name) {
   }
   if (pl.cg == 2) {
     if (g == 2) {
-      // short groups (up to ten k-blocks a tile on average): eight epilogue warps.
-      // GEMM-2's and GEMM-1's weight gradient, four warps -> eight: 136 rows per
-      // expert, D = 2048, F = 1408, E = 60: 154 -> 140 and 273 -> 243 us; 512 rows
-      // (D = 1024, F = 768, E = 256) 204 -> 201 and 373 -> 373; 768 rows (D = 2048,
+      // Very short groups (up to four k-blocks a tile on average), which the fp32
+      // stores bound: the epilogue's stores go through the copy engine, its staging
+      // taking one stage of the ring.  GEMM-2's and GEMM-1's weight gradient at
+      // D = 2048, F = 1408, E = 60 (0.69 and 1.38 GB), stored by eight warps -> by the
+      // copy engine: 17 rows per expert 133 -> 121 and 234 -> 215 us, 136 rows 138 ->
+      // 126 and 244 -> 232, 256 rows 146 -> 136 and 255 -> 248, 384 rows 156 -> 156
+      // and 276 -> 295 (the loads miss the stage).
+      if (d.offsets && d.max_rows <= 4 * (int64_t)tc::BK * d.num_groups && d.M % 64 == 0 && d.N % 64 == 0 &&
+          d.sc_g % 4 == 0 && make_store_map(&p.tc, d))
+        return launch_inst<256, true, true, 2, 0, float, 2, 0, tc::kBulkEpi>(c, p, ub);
+      // Short groups (up to ten): eight epilogue warps.  Four warps -> eight: 512
+      // rows (D = 1024, F = 768, E = 256) 204 -> 201 and 373 -> 373 us, 546 rows
+      // (D = 1408, F = 704, E = 60) 73 -> 72 and 136 -> 130; 768 rows (D = 2048,
       // F = 1024, E = 64) 157 -> 160 and 299 -> 305.
       if (d.offsets && d.max_rows <= 10 * (int64_t)tc::BK * d.num_groups)
         return launch_inst<256, true, true, 2, 0, float, 2, 0, 8>(c, p, ub);

@@ -41,6 +41,7 @@ constexpr uint32_t kSuspendNs = 20000;  // a try sleeps up to this long for its 
 struct Params {
   CUtensorMap ta;
   CUtensorMap tb;
+  CUtensorMap tc;         // Group::K, bulk stores: C as [group][m][n], boxes of 32 x 32
   CUtensorMap ta16;       // Group::M: A in boxes of kARowStep rows (short tiles)
   int64_t M, N, K;
   int64_t b_group_rows;   // rows of B's tensor map per group (Group::M)
@@ -167,6 +168,18 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y)
       : "memory");
 }
+// 32 x 32 fp32 of C from shared memory (128-byte swizzle) to global memory; one
+// bulk group per store.
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(src), "r"(x), "r"(y), "r"(z)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+// Until this thread's bulk stores have read their sources, or have finished.
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
@@ -390,6 +403,10 @@ __host__ __device__ constexpr uint32_t make_idesc(int bn, int bm, bool a_mn, boo
          ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(bm >> 4) << 24);
 }
 
+// The fp32 epilogue (EWF): 4 or 8 warps that stage and store, or kBulkEpi: 8 that
+// hand their chunks to the copy engine.
+constexpr int kBulkEpi = 9;
+
 // CG = 1: one CTA computes a 128 x BN tile.  CG = 2: a cluster of two CTAs
 // computes a 256 x BN tile; each CTA stages its 128 rows of A and BN / 2 rows
 // of B, and holds its 128 accumulator rows in its own TMEM.
@@ -399,24 +416,28 @@ struct Cfg {
   static constexpr int kABytes = BM * BK * 2;
   static constexpr int kBBytes = kBRows * BK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  // EPI 5 (SwiGLU backward) gives one stage to its h slots
-  static constexpr int kStages = EPI == 5 ? 5 : ((196608 / kStageBytes) < 8 ? (196608 / kStageBytes) : 8);
+  // Bulk-store epilogue (weight gradients of short groups, EWF = 8)
+  static constexpr bool kBulk = TCB == 4 && EWF == kBulkEpi;
+  // EPI 5 (SwiGLU backward) gives one stage to its h slots, the bulk-store
+  // epilogue one to its staging
+  static constexpr int kStages = EPI == 5 || kBulk ? 5 : ((196608 / kStageBytes) < 8 ? (196608 / kStageBytes) : 8);
   static constexpr int kCols = 2 * BN;  // double-buffered fp32 accumulator
   // Epilogue warps: 8 (two per TMEM lane quarter, each taking half the
   // columns) for bf16 outputs, whose epilogues are latency-bound; EWF for fp32
   // outputs: 4, which are bound by their store bandwidth beside a long main
   // loop, or 8 where a tile has few k-blocks and its stores are what it takes.
-  static constexpr int kEpiWarps = TCB == 2 ? 8 : EWF;
+  static constexpr int kEpiWarps = TCB == 2 || EWF == kBulkEpi ? 8 : EWF;
   // ZW: one more warp that writes the empty groups' zero gradients (Group::K, fp32)
   static constexpr int kThreads = 64 + 32 * kEpiWarps + 32 * ZW;
   // per epilogue warp: 32 rows x 32 columns of C staging, rows padded by 16 B
-  // (conflict-free both ways); eight warps of fp32 rows stage 16 rows at a time
+  // (conflict-free both ways); eight warps of fp32 rows stage 16 rows at a time;
+  // for a bulk store 32 swizzled 128-byte rows (4 KB)
   static constexpr int kStageRows = TCB == 4 && kEpiWarps == 8 ? 16 : 32;
   static constexpr int kRowBytes = 32 * TCB;
   static constexpr int kPitch = kRowBytes + 16;
   // EPI 5: a ring of three 2 KB slots per warp, each the gate and up blocks of
   // h (in) and of dH (out) for 16 columns of dA, 32 rows x 32 bytes apiece
-  static constexpr int kStageBufBytes = EPI == 5 ? 6144 : kStageRows * kPitch;
+  static constexpr int kStageBufBytes = EPI == 5 ? 6144 : kBulk ? 4096 : kStageRows * kPitch;
   static constexpr int kStagingBytes = kEpiWarps * kStageBufBytes;
   static constexpr int kSmem = kStages * kStageBytes + kStagingBytes + 1024 /*align*/ + 512 /*barriers*/;
 };
@@ -1221,6 +1242,13 @@ __global__ void __launch_bounds__(
       uint8_t* c_rows = reinterpret_cast<uint8_t*>(Cb) + rbase * ldc_b;
       if (ti.nkb == 0) {
         // an expert with no rows: its weight-gradient tile is zero
+        if (C::kBulk) {
+          for (int c = ch; c < BN / 32; c += CSTEP) {
+            const int64_t col = n0 + c * 32 + lane;
+            for (int r = 0; r < nrows && col < p.N; ++r) Cb[(rbase + r) * p.ldc + col] = from_f32<TC>(0.f);
+          }
+          continue;
+        }
         uint4 z[NP];
 #pragma unroll
         for (int i = 0; i < NP; ++i) z[i] = make_uint4(0, 0, 0, 0);
@@ -1381,6 +1409,37 @@ __global__ void __launch_bounds__(
             stage_store<RB>(stg, lane, c_rows + col0 * sizeof(TC), ldc_b, nrows);
           }
         }
+      } else if constexpr (C::kBulk) {
+        // each warp stages 32 x 32 of C, swizzled, and one lane hands it to the copy
+        // engine: the LSU sees one shared store per 16 bytes instead of a store, a
+        // load and a global store.  Rows past M and columns past N are whole chunks
+        // (M and N are multiples of 64 where this is chosen).
+        constexpr int NC = BN / 32 / CSTEP;
+        const int nch = (int)imin64(BN / 32, (p.N - n0) / 32);
+        const uint32_t sbuf = smem_u32(stg);
+        uint32_t ra[32], rb[32];
+        auto put = [&](const uint32_t(&r)[32], int c) {
+          if (elect_one()) tma_store_wait_read();
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            sts128(sbuf + lane * 128 + ((j ^ (lane & 7)) << 4),
+                   make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]));
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (nrows > 0 && elect_one()) tma_store_3d(&p.tc, sbuf, (int)n0 + c * 32, (int)rbase, ti.g);
+        };
+        tmem_ld32_issue(tbase + ch * 32, ra);
+#pragma unroll 1
+        for (int i = 0; i < NC; i += 2) {
+          const int c0 = ch + i * CSTEP, c1 = c0 + CSTEP;
+          tmem_ld_wait(ra);
+          tmem_ld32_issue(tbase + c1 * 32, rb);
+          if (c0 < nch) put(ra, c0);
+          tmem_ld_wait(rb);
+          if (i + 2 < NC) tmem_ld32_issue(tbase + (c1 + CSTEP) * 32, ra);
+          if (c1 < nch) put(rb, c1);
+        }
       } else if (EPI == 0 && n0 + BN <= p.N) {
         // every column of the tile exists: chunk i + 1's TMEM load is in
         // flight while chunk i is staged and stored
@@ -1461,6 +1520,11 @@ __global__ void __launch_bounds__(
         else mbar_arrive(smem_u32(&tempty[acc]));
       }
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+    }
+    if (C::kBulk) {  // the stores have left shared memory, and are done, before the CTA exits
+      __syncwarp();
+      if (elect_one()) tma_store_wait_all();
+      __syncwarp();
     }
     if (EPI == 5) cp_async_wait_all();  // no h copy is still landing when the CTA exits
   }
