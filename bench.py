@@ -65,6 +65,7 @@ def kernel_work(name: str, w: synth.Workload, T: int, Fs: int = 0, latent_fused:
         "shared_fc1": 2.0 * T * Din * Fs, "shared_fc2": 2.0 * T * Fs * Din,
         "shared_fc2_dgrad": 2.0 * T * Din * Fs, "shared_fc1_dgrad": 2.0 * T * Fs * Din,
         "shared_fc2_wgrad": 2.0 * T * Din * Fs, "shared_fc1_wgrad": 2.0 * T * Fs * Din,
+        "shared_wgrad": 4.0 * T * Din * Fs,
     }
     if base in flops:
         return "tensor", flops[base]
@@ -121,6 +122,7 @@ def gemm_bytes(name: str, w: synth.Workload, T: int, Fs: int = 0, latent_fused: 
         "shared_fc1_dgrad": (T * Fs + Fs * Din + 2 * T * Din) * bx,
         "shared_fc2_wgrad": (T * Din + T * Fs) * bx + Din * Fs * 4,
         "shared_fc1_wgrad": (T * Fs + T * Din) * bx + Fs * Din * 4,
+        "shared_wgrad": 2 * ((T * Fs + T * Din) * bx + Fs * Din * 4),
     }
     return float(table.get(base, 0.0))
 

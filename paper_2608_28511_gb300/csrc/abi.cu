@@ -1240,10 +1240,17 @@ int moe_shared_expert_bwd(const moe_shape_t* shape, int32_t F_s, const void* dy,
   // dw_s2 = dy^T . a   (M = Din, N = F_s, K = T)
   GemmDesc w2 = dense_desc(Epi::Store, d.Din, F_s, d.T, dy, d.dt, 1, d.Din, act_save, d.dt, 1, F_s, dw_s2,
                            DType::F32, F_s);
-  TRY_CUDA(gemm(c, w2, "shared_fc2_wgrad_tc", "shared_fc2_wgrad_simt"));
   // dw_s1 = dh^T . x   (M = F_s, N = Din, K = T)
   GemmDesc w1 = dense_desc(Epi::Store, F_s, d.Din, d.T, dh, d.dt, 1, F_s, x, d.dt, 1, d.Din, dw_s1, DType::F32,
                            d.Din);
+  if (gemm_tc_pairable(w2, w1)) {
+    // both weight gradients' tiles in one launch: Din = 2048, F_s = 2688 is 88
+    // tiles each, two rounds of the SM pairs apiece but three together (step of
+    // T = 8192 2144 -> 2125 us)
+    TRY_CUDA(launch_gemm_tc(c, w2, "shared_wgrad_tc", &w1));
+    return MOE_OK;
+  }
+  TRY_CUDA(gemm(c, w2, "shared_fc2_wgrad_tc", "shared_fc2_wgrad_simt"));
   TRY_CUDA(gemm(c, w1, "shared_fc1_wgrad_tc", "shared_fc1_wgrad_simt"));
   return MOE_OK;
 }

@@ -254,7 +254,14 @@ bool gemm_tc_supports(const GemmDesc& d) {
   return false;
 }
 
-cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name) {
+bool gemm_tc_pairable(const GemmDesc& d, const GemmDesc& d2) {
+  Plan a, b;
+  return d.group == Group::Dense && d2.group == Group::Dense && d.epi == Epi::Store && d2.epi == Epi::Store &&
+         gemm_tc_supports(d) && gemm_tc_supports(d2) && make_plan(d, &a) && make_plan(d2, &b) && a.a_mn && a.b_mn &&
+         b.a_mn && b.b_mn && a.cg == b.cg && d.K == d2.K && d.c_type == d2.c_type;
+}
+
+cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name, const GemmDesc* second) {
   Plan pl;
   if (!make_plan(d, &pl) || !gemm_tc_supports(d)) return cudaErrorNotSupported;
   Params p;
@@ -304,8 +311,23 @@ cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name) {
     p.gsrc_ld = pl.ldb * 2;
     p.gsrc_rows = d.gather_rows;
   }
+  p.tiles1 = p.tiles_m * p.tiles_n;
+  if (second) {
+    const GemmDesc& d2 = *second;
+    Plan pl2;
+    if (!gemm_tc_pairable(d, d2) || !make_plan(d2, &pl2)) return cudaErrorNotSupported;
+    if (!make_map(&p.ta2, d2.A, d2.M, d2.K, pl2.lda * 2, 64, 64) ||
+        !make_map(&p.tb2, d2.B, d2.N, d2.K, pl2.ldb * 2, 64, 64))
+      return cudaErrorInvalidValue;
+    p.tiles_n2 = (int)((d2.N + bn - 1) / bn);
+    p.tiles2 = (int)((d2.M + bmp - 1) / bmp) * p.tiles_n2;
+    p.M2 = d2.M;
+    p.N2 = d2.N;
+    p.ldc2 = d2.ldc;
+    p.C2 = d2.C;
+  }
   int64_t ub;
-  if (d.group == Group::Dense) ub = (int64_t)p.tiles_m * p.tiles_n;
+  if (d.group == Group::Dense) ub = (int64_t)p.tiles1 + p.tiles2;
   else if (d.group == Group::M) ub = ((d.max_rows + bmp - 1) / bmp + d.num_groups) * p.tiles_n;
   else ub = (int64_t)d.num_groups * p.tiles_m * p.tiles_n;
   if (ub <= 0) return cudaSuccess;

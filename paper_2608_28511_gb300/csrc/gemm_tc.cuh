@@ -59,6 +59,12 @@ struct Params {
                              // [lo(g), lo(g + 1)), lo(g) = split_rows g / G rounded down to a
                              // multiple of BK (lo(G) = split_rows): only the last split can
                              // end inside a k-block
+  // Dense with both operands MN-major: a second product over the same K, whose
+  // tiles follow the first one's (tiles1 of them; all of them without a second)
+  CUtensorMap ta2, tb2;
+  int tiles1, tiles2, tiles_n2;
+  int64_t M2, N2, ldc2;
+  void* C2;
   const int32_t* gather;     // GATHER: source row of each gathered row (the permutation's token_of_row)
   const uint8_t* gsrc;       // GATHER: the source matrix (bf16, row-major), its row pitch in bytes
   int64_t gsrc_ld;           //   and its row count (source rows are checked against it)
@@ -552,10 +558,14 @@ __device__ __forceinline__ void decode_tile(const Params& p, int t, const int* s
                                             uint32_t rank, Tile& ti) {
   constexpr int BMP = BM * CG;
   if (GROUP == 0) {
-    const int mt = t / p.tiles_n, nt = t % p.tiles_n;
-    ti.g = 0;
+    const bool second = t >= p.tiles1;
+    if (second) t -= p.tiles1;
+    const int tn = second ? p.tiles_n2 : p.tiles_n;
+    const int64_t M = second ? p.M2 : p.M;
+    const int mt = t / tn, nt = t % tn;
+    ti.g = second ? 1 : 0;
     ti.row0 = ((int64_t)mt * CG + rank) * p.tile_rows;
-    ti.row_end = p.M < ti.row0 + p.tile_rows ? p.M : ti.row0 + p.tile_rows;
+    ti.row_end = M < ti.row0 + p.tile_rows ? M : ti.row0 + p.tile_rows;
     ti.n0 = nt;
     ti.kbeg = 0;
     ti.kend = p.K;
@@ -722,6 +732,7 @@ __global__ void __launch_bounds__(
   constexpr int BMP = BM * CG;
   constexpr int BNC = C::kBRows;
   constexpr uint32_t kIdesc = make_idesc(BN, BMP, A_MN, B_MN);
+  constexpr bool kTwo = GROUP == 0 && A_MN && B_MN;  // may carry a second product
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes + C::kStagingBytes);
@@ -848,7 +859,7 @@ __global__ void __launch_bounds__(
   }
   if (tid == 0) {
     if (GROUP == 0) {
-      s_total = p.tiles_m * p.tiles_n;
+      s_total = p.tiles1 + p.tiles2;
     } else if (GROUP == 1) {
       int acc = 0;
       for (int g = 0; g < p.num_groups; ++g) {
@@ -1057,17 +1068,19 @@ __global__ void __launch_bounds__(
             for (int j = 0; j < BNC / 64; ++j) load(sb + j * 8192, mb, (int)nb + 64 * j, ky);
           } else {
             if (A_MN) {
-              load(sa, &p.ta, (int)ti.row0, k0);
-              load(sa + 8192, &p.ta, (int)ti.row0 + 64, k0);
+              const CUtensorMap* ma = kTwo && ti.g ? &p.ta2 : &p.ta;
+              load(sa, ma, (int)ti.row0, k0);
+              load(sa + 8192, ma, (int)ti.row0 + 64, k0);
             } else if (GROUP == 0 || arows == BM) {
               load(sa, &p.ta, k0, (int)ti.row0);
             } else {
               for (int r = 0; r < arows; r += kARowStep) load(sa + r * BK * 2, &p.ta16, k0, (int)ti.row0 + r);
             }
             if (B_MN) {
-              const int ky = (int)(ti.g * p.b_group_rows) + k0;
+              const CUtensorMap* mb = kTwo && ti.g ? &p.tb2 : &p.tb;
+              const int ky = (kTwo ? 0 : (int)(ti.g * p.b_group_rows)) + k0;
 #pragma unroll
-              for (int j = 0; j < BNC / 64; ++j) load(sb + j * 8192, &p.tb, (int)nb + 64 * j, ky);
+              for (int j = 0; j < BNC / 64; ++j) load(sb + j * 8192, mb, (int)nb + 64 * j, ky);
             } else {
               load(sb, &p.tb, k0, (int)(ti.g * p.b_group_rows + nb));
             }
@@ -1225,7 +1238,6 @@ __global__ void __launch_bounds__(
     constexpr int NP = RB / 16;                    // 16-byte pieces per staged row
     constexpr int RPC = (int)sizeof(TC) * 32 / RB; // rounds per 32-column chunk (1)
     constexpr int CPR = RB / (int)sizeof(TC);      // columns per round
-    const int64_t ldc_b = p.ldc * (int64_t)sizeof(TC);
     int acc = 0;
     uint32_t acc_phase = 0;
     int hq = 0;  // EPI 5: ring slot of the current tile's first half
@@ -1238,14 +1250,16 @@ __global__ void __launch_bounds__(
       const int nrows = (int)imax64(0, imin64(32, ti.row_end - rbase));
       const int64_t grow = rbase + lane;
       const bool vrow = lane < nrows;
-      TC* Cb = static_cast<TC*>(p.C) + (GROUP == 2 ? (int64_t)ti.g * p.sc_g : 0);
+      const int64_t N = kTwo && ti.g ? p.N2 : p.N, ldc = kTwo && ti.g ? p.ldc2 : p.ldc;
+      const int64_t ldc_b = ldc * (int64_t)sizeof(TC);
+      TC* Cb = static_cast<TC*>(kTwo && ti.g ? p.C2 : p.C) + (GROUP == 2 ? (int64_t)ti.g * p.sc_g : 0);
       uint8_t* c_rows = reinterpret_cast<uint8_t*>(Cb) + rbase * ldc_b;
       if (ti.nkb == 0) {
         // an expert with no rows: its weight-gradient tile is zero
         if (C::kBulk) {
           for (int c = ch; c < BN / 32; c += CSTEP) {
             const int64_t col = n0 + c * 32 + lane;
-            for (int r = 0; r < nrows && col < p.N; ++r) Cb[(rbase + r) * p.ldc + col] = from_f32<TC>(0.f);
+            for (int r = 0; r < nrows && col < N; ++r) Cb[(rbase + r) * ldc + col] = from_f32<TC>(0.f);
           }
           continue;
         }
@@ -1254,8 +1268,8 @@ __global__ void __launch_bounds__(
         for (int i = 0; i < NP; ++i) z[i] = make_uint4(0, 0, 0, 0);
         for (int c = ch; c < BN / 32; c += CSTEP) {
           const int64_t col0 = n0 + c * 32;
-          if (col0 >= p.N) break;
-          if (p.N - col0 >= 32) {
+          if (col0 >= N) break;
+          if (N - col0 >= 32) {
 #pragma unroll
             for (int r = 0; r < RPC; ++r) {
               stage_rows<RB, C::kStageRows>(stg, lane, z, c_rows + (col0 + r * CPR) * sizeof(TC), ldc_b, nrows);
@@ -1264,7 +1278,7 @@ __global__ void __launch_bounds__(
             float zf[32];
 #pragma unroll
             for (int i = 0; i < 32; ++i) zf[i] = 0.f;
-            store_row32<TC>(Cb + grow * p.ldc + col0, zf, (int)(p.N - col0));
+            store_row32<TC>(Cb + grow * ldc + col0, zf, (int)(N - col0));
           }
         }
         continue;
@@ -1273,7 +1287,7 @@ __global__ void __launch_bounds__(
       // the reads overlap the MMA and each other
       constexpr int kPre = EPI == 2 ? BN / 32 / CSTEP : 1;  // this warp's chunks: ch, ch + CSTEP, ...
       uint4 pre[kPre][4];
-      const int nch_acc = (int)imin64(BN / 32, (p.N - n0) / 32);
+      const int nch_acc = (int)imin64(BN / 32, (N - n0) / 32);
       if (EPI == 2) {
 #pragma unroll
         for (int i = 0; i < kPre; ++i)
@@ -1306,13 +1320,13 @@ __global__ void __launch_bounds__(
       uint4 pk[NP];
       if (EPI == 3) {
         // packed [gate 64 | up 64] blocks: h = [g | u] stored as computed, a = silu(g) * u
-        uint8_t* a_rows = reinterpret_cast<uint8_t*>(static_cast<TC*>(p.aux) + rbase * (p.N / 2));
-        const int64_t lda_b = (p.N / 2) * (int64_t)sizeof(TC);
+        uint8_t* a_rows = reinterpret_cast<uint8_t*>(static_cast<TC*>(p.aux) + rbase * (N / 2));
+        const int64_t lda_b = (N / 2) * (int64_t)sizeof(TC);
 #pragma unroll 1
         for (int hb = ch; hb < BN / 64; hb += CSTEP) {  // half-blocks: 32 gate + 32 up columns
           const int blk = hb >> 1, half = hb & 1;
           const int64_t cb = n0 + blk * 128;
-          if (cb >= p.N) break;
+          if (cb >= N) break;
           {
             // g (in v) and u are stored first; a = silu(g) * u then overwrites v,
             // so only two 32-value rows are live at a time
@@ -1415,7 +1429,7 @@ __global__ void __launch_bounds__(
         // load and a global store.  Rows past M and columns past N are whole chunks
         // (M and N are multiples of 64 where this is chosen).
         constexpr int NC = BN / 32 / CSTEP;
-        const int nch = (int)imin64(BN / 32, (p.N - n0) / 32);
+        const int nch = (int)imin64(BN / 32, (N - n0) / 32);
         const uint32_t sbuf = smem_u32(stg);
         uint32_t ra[32], rb[32];
         auto put = [&](const uint32_t(&r)[32], int c) {
@@ -1440,7 +1454,7 @@ __global__ void __launch_bounds__(
           if (i + 2 < NC) tmem_ld32_issue(tbase + (c1 + CSTEP) * 32, ra);
           if (c1 < nch) put(rb, c1);
         }
-      } else if (EPI == 0 && n0 + BN <= p.N) {
+      } else if (EPI == 0 && n0 + BN <= N) {
         // every column of the tile exists: chunk i + 1's TMEM load is in
         // flight while chunk i is staged and stored
         constexpr int NC = BN / 32 / CSTEP;  // this warp's chunks: ch, ch + CSTEP, ...
@@ -1467,9 +1481,9 @@ __global__ void __launch_bounds__(
 #pragma unroll 1
         for (int c = ch; c < BN / 32; c += CSTEP) {
           const int64_t col0 = n0 + c * 32;
-          if (col0 >= p.N) break;
+          if (col0 >= N) break;
           tmem_ld32(tbase + c * 32, v);
-          const int nvalid = (int)imin64(32, p.N - col0);
+          const int nvalid = (int)imin64(32, N - col0);
           if (EPI == 1 && p.bias) {
 #pragma unroll
             for (int i = 0; i < 32; ++i)
@@ -1478,7 +1492,7 @@ __global__ void __launch_bounds__(
           if (nvalid < 32) {
             // ragged columns: direct row stores
             if (!vrow) continue;
-            TC* crow = Cb + grow * p.ldc;
+            TC* crow = Cb + grow * ldc;
             if (EPI == 2) {
 #pragma unroll
               for (int i = 0; i < 32; ++i)
@@ -1488,7 +1502,7 @@ __global__ void __launch_bounds__(
             if (EPI == 4) {
 #pragma unroll
               for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i], 0.f) * fmaxf(v[i], 0.f);
-              store_row32<TC>(static_cast<TC*>(p.aux) + grow * p.ldc + col0, v, nvalid);
+              store_row32<TC>(static_cast<TC*>(p.aux) + grow * ldc + col0, v, nvalid);
             }
           } else if (EPI == 0 || EPI == 1 || EPI == 4) {
 #pragma unroll

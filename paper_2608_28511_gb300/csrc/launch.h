@@ -175,7 +175,10 @@ cudaError_t launch_gemm_simt_f32x3(const Ctx& c, const GemmDesc (&ds)[3], const 
 // for a descriptor it does not handle.
 bool gemm_tc_supports(const GemmDesc& d);
 size_t gemm_tc_group_scratch_bytes(int num_groups);
-cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name);
+// `second`: another dense product (gemm_tc_pairable: both with MN-major operands
+// over the same K) whose tiles run behind d's in the same launch.
+bool gemm_tc_pairable(const GemmDesc& d, const GemmDesc& second);
+cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name, const GemmDesc* second = nullptr);
 // Builds the per-group tail maps of two Group::K GEMMs over the same groups
 // (the two expert weight gradients) in one launch, into d0.scratch and
 // d1.scratch.  Returns false, launching nothing, unless both are tensor-core

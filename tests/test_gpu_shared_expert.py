@@ -118,3 +118,26 @@ def test_shared_expert_shape_errors():
     with pytest.raises(abi.MoeError) as e:
         abi.moe_shared_expert(L.shape, Fs, L.x, None, L.w_s2, L.h_s, L.act_s, L.y)
     assert e.value.status == -4
+
+
+@pytest.mark.parametrize("Din,Fs,T", [(64, 64, 65), (128, 192, 200), (192, 128, 64), (256, 320, 1000),
+                                      (576, 1088, 333), (1088, 640, 2049)])
+def test_paired_weight_gradients(Din, Fs, T):
+    """Both weight gradients, in one launch where both have tiles of the same
+    height and apart where they have not, at widths that end inside a tile,
+    against float64 from the GPU's own dh and a: sums of T products of bf16
+    values in fp32 stay within about sqrt(T) 2^-24 of the norm, of which four
+    times is allowed."""
+    from paper_2608_28511_gb300 import abi
+    g = torch.Generator(device="cuda").manual_seed(T)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()  # noqa: E731
+    shp = abi.MoeShape.of(T, 1, 1, Din, 1, 64, "bf16")
+    dy, x, h, act, ws1, ws2 = rnd(T, Din), rnd(T, Din), rnd(T, Fs), rnd(T, Fs), rnd(Fs, Din), rnd(Din, Fs)
+    dh, dx = torch.empty_like(h), torch.zeros_like(x)
+    d1, d2 = torch.full((Fs + 1, Din), 3.0, device="cuda"), torch.full((Din + 1, Fs), 3.0, device="cuda")
+    abi.moe_shared_expert_bwd(shp, Fs, dy, x, h, act, ws1, ws2, dh, dx, d1[:Fs], d2[:Din])
+    assert abi.moe_check_device_status() == 0
+    assert bool((d1[Fs] == 3.0).all()) and bool((d2[Din] == 3.0).all())
+    tol = 4.0 * max(T, 16) ** 0.5 * 2.0 ** -24
+    for got, ref in ((d1[:Fs], dh.double().T @ x.double()), (d2[:Din], dy.double().T @ act.double())):
+        assert float((got.double() - ref).norm() / ref.norm()) < tol
