@@ -287,6 +287,8 @@ cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name, co
   const int64_t b_inner = pl.b_mn ? d.N : d.K;
   if (!make_map(&p.tb, d.B, b_inner, b_rows, pl.ldb * 2, 64, gb ? 1 : (pl.b_mn ? 64 : bnc)))
     return cudaErrorInvalidValue;
+  if (!pl.b_mn && !gb && pl.cg == 2 && !make_map(&p.tb64, d.B, b_inner, b_rows, pl.ldb * 2, 64, 64))
+    return cudaErrorInvalidValue;
   p.M = d.M;
   p.N = d.N;
   p.K = d.K;

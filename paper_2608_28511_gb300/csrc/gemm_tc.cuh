@@ -41,6 +41,7 @@ constexpr uint32_t kSuspendNs = 20000;  // a try sleeps up to this long for its 
 struct Params {
   CUtensorMap ta;
   CUtensorMap tb;
+  CUtensorMap tb64;       // K-major B of a CTA pair in boxes of 64 rows (half-width tiles)
   CUtensorMap tc;         // Group::K, bulk stores: C as [group][m][n], boxes of 32 x 32
   CUtensorMap ta16;       // Group::M: A in boxes of kARowStep rows (short tiles)
   int64_t M, N, K;
@@ -596,6 +597,16 @@ __device__ __forceinline__ void decode_tile(const Params& p, int t, const int* s
   ti.nkb = (int)((ti.kend - ti.kbeg + BK - 1) / BK);
 }
 
+// A CTA pair's last column tile with at most BN / 2 columns is computed and its B
+// copied at half width (N = 128 MMAs; each CTA's 64 rows of B).  At D = 1408,
+// F = 704, T = 8191, E = 60, where four of the six expert GEMMs have 5.5 column
+// tiles, the block takes 659 -> 645 us, most of it from the lower power draw; the
+// bulk-store weight gradients, which are bound by their stores, are left alone.
+template <int BN>
+__device__ __forceinline__ bool half_width(const Params& p, const Tile& ti, bool two) {
+  return (two && ti.g ? p.N2 : p.N) - ti.n0 * BN <= BN / 2;
+}
+
 // The tiles one walker (a CTA, or a CTA pair) takes, in order.  Dense and
 // Group::M GEMMs: tiles cta0, cta0 + ncta, ...  Group::K GEMMs (per-expert
 // weight gradients) cost in proportion to the group's rows, and a group
@@ -733,6 +744,7 @@ __global__ void __launch_bounds__(
   constexpr int BNC = C::kBRows;
   constexpr uint32_t kIdesc = make_idesc(BN, BMP, A_MN, B_MN);
   constexpr bool kTwo = GROUP == 0 && A_MN && B_MN;  // may carry a second product
+  constexpr bool kHalf = CG == 2 && BN == 256 && GATHER == 0 && EPI != 1 && !C::kBulk;  // half-width last column tiles
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes + C::kStagingBytes);
@@ -1029,7 +1041,8 @@ __global__ void __launch_bounds__(
       for (int t; ok && next_tile<GROUP>(wk, s_off, s_pref, t);) {
         Tile ti;
         decode_tile<GROUP, CG>(p, t, s_off, s_pref, rank, ti);
-        const int64_t nb = ti.n0 * BN + (int64_t)rank * BNC;  // this CTA's first B row / column
+        const bool half = kHalf && half_width<BN>(p, ti, kTwo);
+        const int64_t nb = ti.n0 * BN + (int64_t)rank * (half ? 64 : BNC);  // this CTA's first B row / column
         // Group::M: the A rows that exist (kAShort); the leader expects both CTAs' copies
         const int arows = GROUP == 1 ? a_rows_copied(ti.row0, ti.row_end) : GROUP == 0 ? p.tile_rows : BM;
         const int abytes =
@@ -1039,7 +1052,7 @@ __global__ void __launch_bounds__(
           const uint32_t fb_local = smem_u32(&full[stage]);
           // CG 2: both CTAs' copies complete on the leader's barrier, which expects both
           const uint32_t fb = CG == 2 ? map_to_rank(fb_local, 0) : fb_local;
-          if (leader) mbar_expect_tx(fb_local, CG * C::kBBytes + abytes);
+          if (leader) mbar_expect_tx(fb_local, CG * (half ? C::kBBytes / 2 : C::kBBytes) + abytes);
           const uint32_t sa = smem_u32(smem + stage * C::kStageBytes);
           const uint32_t sb = sa + C::kABytes;
           const int k0 = (int)(ti.kbeg + (int64_t)kb * BK);
@@ -1065,7 +1078,8 @@ __global__ void __launch_bounds__(
             load(sa, ma, (int)ti.row0, ky);
             load(sa + 8192, ma, (int)ti.row0 + 64, ky);
 #pragma unroll
-            for (int j = 0; j < BNC / 64; ++j) load(sb + j * 8192, mb, (int)nb + 64 * j, ky);
+            for (int j = 0; j < BNC / 64; ++j)
+              if (j == 0 || !half) load(sb + j * 8192, mb, (int)nb + 64 * j, ky);
           } else {
             if (A_MN) {
               const CUtensorMap* ma = kTwo && ti.g ? &p.ta2 : &p.ta;
@@ -1080,9 +1094,10 @@ __global__ void __launch_bounds__(
               const CUtensorMap* mb = kTwo && ti.g ? &p.tb2 : &p.tb;
               const int ky = (kTwo ? 0 : (int)(ti.g * p.b_group_rows)) + k0;
 #pragma unroll
-              for (int j = 0; j < BNC / 64; ++j) load(sb + j * 8192, mb, (int)nb + 64 * j, ky);
+              for (int j = 0; j < BNC / 64; ++j)
+                if (j == 0 || !half) load(sb + j * 8192, mb, (int)nb + 64 * j, ky);
             } else {
-              load(sb, &p.tb, k0, (int)(ti.g * p.b_group_rows + nb));
+              load(sb, half ? &p.tb64 : &p.tb, k0, (int)(ti.g * p.b_group_rows + nb));
             }
           }
           last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
@@ -1135,6 +1150,8 @@ __global__ void __launch_bounds__(
         if (!wait_bounded(smem_u32(&tempty[acc]), acc_phase ^ 1u, &s_abort, p.err)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+        const uint32_t idesc =
+            kHalf && half_width<BN>(p, ti, kTwo) ? make_idesc(BN / 2, BMP, A_MN, B_MN) : kIdesc;
         for (int kb = 0; kb < ti.nkb; ++kb) {
           if (!wait_bounded(smem_u32(&full[stage]), phase, &s_abort, p.err, GATHER != 0 && CG == 2)) {
             ok = false;
@@ -1147,7 +1164,7 @@ __global__ void __launch_bounds__(
           const uint64_t bd = make_sdesc(sa + C::kABytes, B_MN ? 8192 : 16, 1024);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)  // 16 elements of k: 32 bytes, or 2048 MN-major, in units of 16
-            mma_bf16_cg<CG>(d_tmem, ad + k * (A_MN ? 128 : 2), bd + k * (B_MN ? 128 : 2), kIdesc,
+            mma_bf16_cg<CG>(d_tmem, ad + k * (A_MN ? 128 : 2), bd + k * (B_MN ? 128 : 2), idesc,
                             (kb > 0 || k > 0) ? 1u : 0u);
           mma_commit_cg<CG>(smem_u32(&empty[stage]), kBoth);
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
