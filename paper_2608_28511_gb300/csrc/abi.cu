@@ -388,9 +388,12 @@ int moe_dispatch(const moe_shape_t* shape, const void* x, const int32_t* topk_id
   if (ws_bytes < ws_perm(d)) return MOE_ERR_WORKSPACE;
   Ctx c;
   TRY(get_ctx(stream, &c));
-  TRY_CUDA(launch_permutation(c, topk_idx, topk_prob, d.T, d.K, d.E, expert_offsets, row_of_slot, token_of_row,
-                              prob_perm, ws));
-  if (x_perm) TRY_CUDA(launch_dispatch_rows(c, x, row_of_slot, d.T, d.K, (int64_t)d.D * d.bx, x_perm));
+  if (x_perm)
+    TRY_CUDA(launch_permute_dispatch(c, x, topk_idx, topk_prob, d.T, d.K, d.E, (int64_t)d.D * d.bx, expert_offsets,
+                                     row_of_slot, token_of_row, prob_perm, x_perm, ws));
+  else
+    TRY_CUDA(launch_permutation(c, topk_idx, topk_prob, d.T, d.K, d.E, expert_offsets, row_of_slot, token_of_row,
+                                prob_perm, ws));
   return MOE_OK;
 }
 

@@ -76,10 +76,10 @@ extern "C" int moe_dispatch_noalloc(const moe_shape_t* shape, const void* x, con
   if (st != MOE_OK) return st;
   // Every table entry the kernels read is written earlier in the same call
   // (the histogram writes all E x chunks counts), so no clearing is needed.
-  st = abi_cuda_status(launch_permutation(c, topk_idx, topk_prob, d.T, d.K, d.E, expert_offsets, row_of_slot,
-                                          token_of_row, prob_perm, scratch));
-  if (st != MOE_OK) return st;
   if (x_perm)
-    st = abi_cuda_status(launch_dispatch_rows(c, x, row_of_slot, d.T, d.K, (int64_t)d.D * d.bx, x_perm));
-  return st;
+    return abi_cuda_status(launch_permute_dispatch(c, x, topk_idx, topk_prob, d.T, d.K, d.E, (int64_t)d.D * d.bx,
+                                                   expert_offsets, row_of_slot, token_of_row, prob_perm, x_perm,
+                                                   scratch));
+  return abi_cuda_status(launch_permutation(c, topk_idx, topk_prob, d.T, d.K, d.E, expert_offsets, row_of_slot,
+                                            token_of_row, prob_perm, scratch));
 }

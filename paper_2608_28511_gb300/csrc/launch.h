@@ -82,6 +82,10 @@ cudaError_t launch_permutation(const Ctx& c, const int32_t* idx, const float* pr
                                void* ws);
 cudaError_t launch_dispatch_rows(const Ctx& c, const void* x, const int32_t* row_of_slot, int64_t T, int K,
                                  int64_t row_bytes, void* x_perm);
+// The permutation and the row copies to x_perm; one launch for up to 512 slots.
+cudaError_t launch_permute_dispatch(const Ctx& c, const void* x, const int32_t* idx, const float* prob, int64_t T,
+                                    int K, int E, int64_t row_bytes, int32_t* offsets, int32_t* row_of_slot,
+                                    int32_t* token_of_row, float* prob_perm, void* x_perm, void* ws);
 cudaError_t launch_combine(const Ctx& c, DType dt, const void* y_perm, const float* prob_perm,
                            const int32_t* row_of_slot, int64_t T, int K, int D, void* y);
 cudaError_t launch_combine_bwd(const Ctx& c, DType dt, const void* dy, const void* y_perm, const float* prob_perm,

@@ -11,6 +11,7 @@ namespace moe {
 constexpr int kChunk = 2048;       // slots per counting-sort chunk
 constexpr int kRankWarps = 8;      // sub-chunks of kChunk / kRankWarps slots
 constexpr int kSub = kChunk / kRankWarps;
+constexpr int kSmallDispatch = 512;  // slots up to which permutation and row copies are one launch
 
 static inline int64_t num_chunks(int64_t TK) { return (TK + kChunk - 1) / kChunk; }
 
@@ -57,15 +58,26 @@ __global__ void __launch_bounds__(256) perm_hist_kernel(const int32_t* __restric
 // writes prob_perm.  Bound by its chain of round trips: 16 of a table column's
 // counts are in flight at once, and one thread per expert scans the totals by
 // shuffles: 64 chunks of E = 256 16.9 -> 10.6 us.
+//
+// COPY (a single chunk): the dispatch itself rides along.  Every block ranks all
+// slots (block 0 writes the arrays) and keeps the rows in shared memory, then the
+// grid's warps copy the tokens' rows of x, a token's row split over eight warps.
+// It saves the second launch and the rows' trip through memory: 512 slots of 4 KB
+// 6.0 -> 5.0 us, 384 slots 6.2 -> 5.1; at 2000 slots the ranking of every block
+// costs more than the launch (7.5 -> 10.7), so up to kSmallDispatch slots.
+template <bool COPY>
 __global__ void __launch_bounds__(kRankWarps * 32) perm_rank_kernel(
     const int32_t* __restrict__ idx, const float* __restrict__ prob, int64_t TK, int K, int E, int nchunks,
     const int32_t* __restrict__ counts, int32_t* __restrict__ offsets, int32_t* __restrict__ row_of_slot,
-    int32_t* __restrict__ token_of_row, float* __restrict__ prob_perm, uint32_t* err) {
+    int32_t* __restrict__ token_of_row, float* __restrict__ prob_perm, uint32_t* err, const uint4* __restrict__ x,
+    int vpr, uint4* __restrict__ x_perm) {
   static_assert(kRankWarps * 32 >= kMaxE, "one thread per expert");
   __shared__ int cnt[kRankWarps * kMaxE];
   __shared__ int wsum[kRankWarps];
+  __shared__ int32_t s_rows[COPY ? kSmallDispatch : 1];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t w0 = (int64_t)blockIdx.x * kChunk + (int64_t)warp * kSub;
+  const bool writes = !COPY || blockIdx.x == 0;
+  const int64_t w0 = (COPY ? 0 : (int64_t)blockIdx.x * kChunk) + (int64_t)warp * kSub;
   const int64_t w1 = min(TK, w0 + kSub);
   // the warp's kSub expert indices and probabilities, all loads in flight at
   // once (expert -1 past the end)
@@ -135,14 +147,29 @@ __global__ void __launch_bounds__(kRankWarps * 32) perm_rank_kernel(
     __syncwarp();
     if (valid) {
       const int row = here + rank;
-      row_of_slot[s] = row;
-      token_of_row[row] = (int32_t)(s / K);
-      prob_perm[row] = pv[i];
+      if (COPY) s_rows[s] = row;
+      if (writes) {
+        row_of_slot[s] = row;
+        token_of_row[row] = (int32_t)(s / K);
+        prob_perm[row] = pv[i];
+      }
       if (rank == __popc(peers) - 1) cnt[warp * E + e] = here + __popc(peers);
     } else if (s < w1) {
-      row_of_slot[s] = 0;  // keeps downstream gathers in bounds; the status word is set
+      if (COPY) s_rows[s] = 0;
+      if (writes) row_of_slot[s] = 0;  // keeps downstream gathers in bounds; the status word is set
     }
     __syncwarp();
+  }
+  if (COPY) {
+    __syncthreads();
+    const int parts = (int)(TK / K) * 8;  // at most 8 kSmallDispatch
+    for (int i = (int)blockIdx.x * kRankWarps + warp; i < parts; i += (int)gridDim.x * kRankWarps) {
+      const int t = i >> 3;
+      for (int v = (i & 7) * 32 + lane; v < vpr; v += 256) {
+        const uint4 val = ld_stream(x + (int64_t)t * vpr + v);
+        for (int k = 0; k < K; ++k) st_stream(x_perm + (int64_t)s_rows[t * K + k] * vpr + v, val);
+      }
+    }
   }
 }
 
@@ -164,8 +191,9 @@ cudaError_t launch_permutation(const Ctx& c, const int32_t* idx, const float* pr
   }
   {
     KernelScope ks("perm_rank", c.stream);
-    perm_rank_kernel<<<nch, kRankWarps * 32, 0, c.stream>>>(idx, prob, TK, K, E, nch, counts, offsets,
-                                                            row_of_slot, token_of_row, prob_perm, c.err);
+    perm_rank_kernel<false><<<nch, kRankWarps * 32, 0, c.stream>>>(idx, prob, TK, K, E, nch, counts, offsets,
+                                                                   row_of_slot, token_of_row, prob_perm, c.err,
+                                                                   nullptr, 0, nullptr);
   }
   return cudaGetLastError();
 }
@@ -196,8 +224,8 @@ static inline int k_bound(int K) { return K <= 2 ? 2 : (K <= 4 ? 4 : (K <= 8 ? 8
 // Warps per token (P): a warp walks its row 32 vectors at a time, and each step
 // is a round trip to memory, so a batch with few rows is bound by that chain.
 // Eight warps share a token's row where fewer than 16 rows per SM are in flight
-// with one warp per token: T = 64, K = 6, D = 2048 dispatch 8.6 -> 3.6 us,
-// combine 9.6 -> 4.1.  Above it is even (8180 rows of 4 KB) or slower (9003 rows
+// with one warp per token: T = 64, K = 6, D = 2048 combine 9.6 -> 4.1 us (row
+// copies alone 8.6 -> 3.6).  Above it is even (8180 rows of 4 KB) or slower (9003 rows
 // of 2 KB: fused dispatch / router backward 8 -> 16 us).
 static inline int row_parts(const Ctx& c, int64_t T, int K, int vpr) {
   return vpr >= 128 && T * K < (int64_t)c.num_sms * 16 ? 8 : 1;
@@ -560,6 +588,24 @@ cudaError_t launch_dispatch_route_bwd(const Ctx& c, DType dt, const void* dx_per
                            E, vpr, (uint4*)dx, dprob, dz, (bf16*)dz16, c.err)));
   }
   return cudaGetLastError();
+}
+
+cudaError_t launch_permute_dispatch(const Ctx& c, const void* x, const int32_t* idx, const float* prob, int64_t T,
+                                    int K, int E, int64_t row_bytes, int32_t* offsets, int32_t* row_of_slot,
+                                    int32_t* token_of_row, float* prob_perm, void* x_perm, void* ws) {
+  const int64_t TK = T * K;
+  if (TK > 0 && TK <= kSmallDispatch) {
+    const unsigned grid = (unsigned)(T < 4 * (int64_t)c.num_sms ? T : 4 * (int64_t)c.num_sms);
+    KernelScope ks("perm_dispatch", c.stream);
+    perm_rank_kernel<true><<<grid, kRankWarps * 32, 0, c.stream>>>(
+        idx, prob, TK, K, E, 1, nullptr, offsets, row_of_slot, token_of_row, prob_perm, c.err, (const uint4*)x,
+        (int)(row_bytes / 16), (uint4*)x_perm);
+    return cudaGetLastError();
+  }
+  const cudaError_t st =
+      launch_permutation(c, idx, prob, T, K, E, offsets, row_of_slot, token_of_row, prob_perm, ws);
+  if (st != cudaSuccess) return st;
+  return launch_dispatch_rows(c, x, row_of_slot, T, K, row_bytes, x_perm);
 }
 
 // w1[e, 128 i + c] = w_gate[e, 64 i + c] for c < 64, w_up[e, 64 i + c - 64] otherwise.
