@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(256) topk_kernel(const float* __restrict__ log
   int me;
   sel::warp_topk<V>(key, E, K, lane, slots[threadIdx.x >> 5], [&] { return row; }, &mk, &me, &best);
   const float w = lane < K ? expf(mk - best) : 0.f;
-  const float inv = 1.0f / sel::sum16(w);
+  const float inv = 1.0f / sel::sum_chosen(w, K);
   if (lane < K) {
     idx[t * K + lane] = me;
     prob[t * K + lane] = w * inv;

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(32 * kSelWarps) select_sigmoid_kernel(
       const float sv = __shfl_sync(0xffffffffu, s[v], me & 31);
       if (me >> 5 == v && lane < K) sk = sv;
     }
-    const float ginv = __frcp_rn(sel::sum16(sk));
+    const float ginv = __frcp_rn(sel::sum_chosen(sk, K));
     if (lane < K) {
       idx[t * K + lane] = me;
       prob[t * K + lane] = sk * ginv;

@@ -146,12 +146,14 @@ __device__ __forceinline__ void warp_topk(float (&key)[V], int E, int K, int lan
   __syncwarp();  // the slots are read before the next token's rounds write them
 }
 
-// The sum of the values of lanes 0 .. 15 (at most 16 experts are chosen; the
-// other lanes pass 0), in every lane.
-__device__ __forceinline__ float sum16(float v) {
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return __shfl_sync(0xffffffffu, v, 0);
+// The sum of the values of lanes 0 .. K - 1, added in that order (best expert
+// first), in every lane: a probability is a function of its chosen keys alone,
+// not of how the lanes are paired.
+__device__ __forceinline__ float sum_chosen(float v, int K) {
+  float s = 0.f;
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) s += __shfl_sync(0xffffffffu, v, k);
+  return s;
 }
 
 }  // namespace sel

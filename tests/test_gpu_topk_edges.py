@@ -41,3 +41,26 @@ def test_selection(E, K):
     w = np.exp(top[fine] - top[fine][:, :1])
     assert np.abs(prob.cpu().numpy()[fine] - w / w.sum(1, keepdims=True)).max() <= 1e-6
     assert abi.moe_check_device_status() == 0
+
+
+@pytest.mark.parametrize("K", [5, 8, 16])
+def test_probabilities_are_summed_best_first(K):
+    """One logit 17 above the others, whose terms (4.1e-8 and less, of a best one
+    of 1) are each below half a unit in the last place of the running sum when
+    added best first: the sum is exactly 1.  Added to each other first they move
+    it.  The same for the sigmoid scores, of which the best is exactly 1."""
+    T, E = 40, 64
+    z = -17.0 - 0.01 * torch.rand(T, E, generator=torch.Generator().manual_seed(K))
+    best = torch.arange(T) % E
+    z[torch.arange(T), best] = 0.0
+    idx = torch.empty(T, K, dtype=torch.int32, device="cuda")
+    prob = torch.empty(T, K, device="cuda")
+    shp = abi.MoeShape.of(T, 1, K, 64, E, 64)
+    abi.moe_topk(shp, z.cuda(), idx, prob)
+    assert torch.equal(idx[:, 0].cpu().long(), best) and bool((prob[:, 0] == 1.0).all())
+    z[torch.arange(T), best] = 40.0
+    f, loss = torch.empty(1, E, device="cuda"), torch.empty(4, device="cuda")
+    ws = torch.empty(abi.moe_workspace_size(shp), dtype=torch.uint8, device="cuda")
+    abi.moe_topk_sigmoid(shp, z.cuda(), None, 1e-4, None, idx, prob, f, loss, ws)
+    assert torch.equal(idx[:, 0].cpu().long(), best) and bool((prob[:, 0] == 1.0).all())
+    assert abi.moe_check_device_status() == 0
