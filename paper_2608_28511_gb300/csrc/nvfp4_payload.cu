@@ -9,6 +9,7 @@
 // q * s_b * g is exact in bf16.
 #include <cuda_fp4.h>
 #include <cuda_fp8.h>
+#include <math_constants.h>
 
 #include "common.cuh"
 #include "launch.h"
@@ -61,8 +62,9 @@ __device__ __forceinline__ uint2 e2m1_codes(const float (&f)[kBlk], Q quot) {
 // exact in fp32) comes out exactly, and any other differs from every midpoint by
 // more than 2^-12 of it (v has 8 significant bits, midpoint times den at most 7):
 // the codes are those of the exact quotient.  T = 8191, K = 6, D = 2048: 23.7 ->
-// 19.3 us.  rl has to be a normal number, so a
-// den outside 2^-100 .. 2^100 takes the division.
+// 19.3 us.  rl has to be a normal number, so a den outside 2^-100 .. 2^100 takes
+// the division, and so does a block with an infinity (inf rh + inf rl is NaN for
+// rl <= 0).  The sign is v's: -0 rh + -0 rl is +0 for rl < 0.
 __device__ __forceinline__ void quantize_block(const uint4& v0, const uint4& v1, float six_g, float g,
                                                uint8_t* scode, uint2* codes) {
   float f[kBlk];
@@ -77,10 +79,10 @@ __device__ __forceinline__ void quantize_block(const uint4& v0, const uint4& v1,
   uint2 w = make_uint2(0u, 0u);
   if (sb > 0.f) {
     const float den = sb * g;  // exact: an E4M3 value times a power of two
-    if (den >= 0x1p-100f && den <= 0x1p100f) {
+    if (den >= 0x1p-100f && den <= 0x1p100f && amax < CUDART_INF_F) {
       const float rh = 1.0f / den;
       const float rl = fmaf(-rh, den, 1.0f) * rh;
-      w = e2m1_codes(f, [&](float v) { return fmaf(v, rh, v * rl); });
+      w = e2m1_codes(f, [&](float v) { return copysignf(fmaf(v, rh, v * rl), v); });
     } else {
       w = e2m1_codes(f, [&](float v) { return v / den; });
     }

@@ -200,3 +200,40 @@ def test_row_widths_around_the_register_path(D):
     rounds of 32 blocks."""
     g = torch.Generator().manual_seed(D)
     _check_direct(torch.randn(37, D, generator=g).to(torch.bfloat16), K=3, E=8)
+
+
+def test_signed_zeros():
+    """Negative zeros keep their sign bit (code 8) under every mantissa of the
+    block scale, among values of both signs."""
+    g = torch.Generator().manual_seed(11)
+    x = torch.randn(48, 192, generator=g) * torch.pow(2.0, torch.linspace(-60, 60, 48)).unsqueeze(1)
+    x[:, ::3] = -0.0
+    x[:, 1::7] = 0.0
+    x[5] = -0.0
+    _check_direct(x.to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("D", [64, 2112])
+def test_infinities_saturate_with_their_sign(D):
+    """Codes against the E2M1 value of x / (s_b g) with the row and block scales
+    that the row was sent with: an infinity saturates to 6 of its own sign, NaN to
+    the largest positive value, and the finite blocks beside them are unchanged."""
+    g = torch.Generator().manual_seed(D)
+    x = torch.randn(16, D, generator=g)
+    inf, nan = float("inf"), float("nan")
+    x[0, 3], x[0, 4], x[1, 17], x[2, 0], x[2, 63] = inf, -inf, -inf, inf, -inf
+    x[3] = -inf
+    x[4, 9], x[4, 30], x[5, 20] = nan, -inf, -nan
+    x = x.to(torch.bfloat16)
+    t, q, bs, rs, _ = _dispatch_nvfp4(x, 2, 8)
+    v = x.float().numpy()[t]
+    lut = np.array([O.e4m3_value(int(c)) for c in range(256)])
+    den = (np.repeat(lut[bs], 16, axis=1) * rs[:, None]).astype(np.float32)
+    blockmax = np.fmax.reduce(np.abs(v).reshape(len(t), -1, 16), axis=2)
+    assert (bs[np.isinf(blockmax)] == 0x7E).all()
+    with np.errstate(all="ignore"):
+        want = O.e2m1_quantize_array((v / den).astype(np.float64))
+    want = np.where(den > 0, np.where(np.isnan(v), 7, want), 0)
+    got = np.empty_like(want)
+    got[:, 0::2], got[:, 1::2] = q & 0xF, q >> 4
+    assert np.array_equal(got, want)
