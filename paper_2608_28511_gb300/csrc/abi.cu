@@ -151,6 +151,11 @@ int check_shape(const moe_shape_t* s, Dims* d) {
 
 bool aligned(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
+// The two buffers share memory.
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  return (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na;
+}
+
 #define REQUIRE_PTR(p)                     \
   do {                                     \
     if (!(p)) return MOE_ERR_NULL;         \
@@ -704,7 +709,13 @@ static int expert_ffn_bwd_impl(const Ctx& c, const Dims& d, const void* dy_perm,
   w.ldc = d.D;
   w.sc_g = (int64_t)2 * d.F * d.D;
   if (d.TK > 0) TRY_CUDA(gemm(c, a, "ffn2_dgrad_swiglu_tc", "ffn2_dgrad_swiglu_simt"));
-  if (d.dt == DType::F32) {
+  // a caller may have dx_perm take the place of a buffer that only the weight
+  // gradients still read
+  const size_t rows = (size_t)d.TK, dx_bytes = rows * d.D * d.bx;
+  const bool dx_apart = !overlap(dx_perm, dx_bytes, dy_perm, dx_bytes) &&
+                        !overlap(dx_perm, dx_bytes, x_rows, (gather ? (size_t)d.T : rows) * d.D * d.bx) &&
+                        !overlap(dx_perm, dx_bytes, act_save, rows * d.F * d.bx);
+  if (d.dt == DType::F32 && dx_apart) {
     // the three products that depend on dH, in one launch: each alone leaves SMs
     // idle on a small batch, and in its last wave on a larger one (T = 256,
     // D = 128, E = 8, K = 2, F = 256: 33 -> 18.5 us; T = 3001, D = 512, E = 12,
@@ -723,7 +734,8 @@ static int expert_ffn_bwd_impl(const Ctx& c, const Dims& d, const void* dy_perm,
   TRY_CUDA(gemm(c, b, "ffn2_wgrad_tc", "ffn2_wgrad_simt"));
   TRY_CUDA(gemm(c, w, "ffn1_wgrad_tc", "ffn1_wgrad_simt"));
   // dgrad-1 last: the dispatch backward that follows reads its output while
-  // part of it is still in L2 (the weight gradients' fp32 writes would flush it)
+  // part of it is still in L2 (the weight gradients' fp32 writes would flush it),
+  // and dx_perm may overwrite what the weight gradients have read
   if (d.TK > 0) TRY_CUDA(gemm(c, cg, "ffn1_dgrad_tc", "ffn1_dgrad_simt"));
   return MOE_OK;
 }

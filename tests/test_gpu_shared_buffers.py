@@ -1,0 +1,41 @@
+"""Calls whose output takes the place of an input that the call has finished
+with: the same bits as with buffers of their own."""
+import itertools
+
+import pytest
+import torch
+
+from paper_2608_28511_gb300 import abi
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("counts,D,F", [([700, 0, 129, 300], 256, 256), ([5] * 40, 128, 128)])
+@pytest.mark.parametrize("over", ["dy_perm", "x_perm", "act"])
+def test_expert_backward_dx_over_an_input(over, counts, D, F, dtype):
+    """moe_expert_ffn_bwd with dx_perm over an input of its size."""
+    E, TK = len(counts), sum(counts)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(TK + D)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").to(dt)  # noqa: E731
+    shp = abi.MoeShape.of(TK, 1, 1, D, E, F, dtype)
+    off = torch.tensor([0] + list(itertools.accumulate(counts)), dtype=torch.int32, device="cuda")
+    inp = {"dy_perm": rnd(TK, D), "x_perm": rnd(TK, D), "h": rnd(TK, 2 * F), "act": rnd(TK, F)}
+    w1, w2 = rnd(E, 2 * F, D), rnd(E, D, F)
+    ws = torch.empty(abi.moe_workspace_size(shp), dtype=torch.uint8, device="cuda")
+    out = []
+    for shared in (False, True):
+        b = {k: v.clone() for k, v in inp.items()}
+        dx = b[over] if shared else torch.empty(TK, D, dtype=dt, device="cuda")
+        dw1, dw2 = torch.empty(E, 2 * F, D, device="cuda"), torch.empty(E, D, F, device="cuda")
+        abi.moe_expert_ffn_bwd(shp, b["dy_perm"], b["x_perm"], b["h"], b["act"], off, w1, w2, dx, dw1, dw2, ws)
+        out.append((dx, dw1, dw2))
+    assert abi.moe_check_device_status() == 0
+    assert all(torch.equal(p, q) for p, q in zip(*out))
