@@ -151,11 +151,6 @@ int check_shape(const moe_shape_t* s, Dims* d) {
 
 bool aligned(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-// The two buffers share memory.
-bool overlap(const void* a, size_t na, const void* b, size_t nb) {
-  return (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na;
-}
-
 #define REQUIRE_PTR(p)                     \
   do {                                     \
     if (!(p)) return MOE_ERR_NULL;         \

@@ -32,6 +32,11 @@ enum class DType : int { BF16 = 0, F32 = 1 };
 
 inline size_t dsize(DType t) { return t == DType::BF16 ? 2 : 4; }
 
+// The two buffers share memory.
+inline bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  return (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na;
+}
+
 // Shape validation and per-device context shared by the entry points
 // (implemented in abi.cu).
 struct ShapeInfo {
@@ -82,7 +87,8 @@ cudaError_t launch_permutation(const Ctx& c, const int32_t* idx, const float* pr
                                void* ws);
 cudaError_t launch_dispatch_rows(const Ctx& c, const void* x, const int32_t* row_of_slot, int64_t T, int K,
                                  int64_t row_bytes, void* x_perm);
-// The permutation and the row copies to x_perm; one launch for up to 512 slots.
+// The permutation and the row copies to x_perm; one launch for up to 512 slots,
+// unless an output lies over idx, which every block of that launch reads.
 cudaError_t launch_permute_dispatch(const Ctx& c, const void* x, const int32_t* idx, const float* prob, int64_t T,
                                     int K, int E, int64_t row_bytes, int32_t* offsets, int32_t* row_of_slot,
                                     int32_t* token_of_row, float* prob_perm, void* x_perm, void* ws);

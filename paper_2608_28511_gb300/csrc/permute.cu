@@ -594,7 +594,11 @@ cudaError_t launch_permute_dispatch(const Ctx& c, const void* x, const int32_t* 
                                     int K, int E, int64_t row_bytes, int32_t* offsets, int32_t* row_of_slot,
                                     int32_t* token_of_row, float* prob_perm, void* x_perm, void* ws) {
   const int64_t TK = T * K;
-  if (TK > 0 && TK <= kSmallDispatch) {
+  const size_t nb = (size_t)TK * 4;
+  const bool idx_apart = !overlap(idx, nb, row_of_slot, nb) && !overlap(idx, nb, token_of_row, nb) &&
+                         !overlap(idx, nb, prob_perm, nb) && !overlap(idx, nb, offsets, (size_t)(E + 1) * 4) &&
+                         !overlap(idx, nb, x_perm, (size_t)TK * row_bytes);
+  if (TK > 0 && TK <= kSmallDispatch && idx_apart) {
     const unsigned grid = (unsigned)(T < 4 * (int64_t)c.num_sms ? T : 4 * (int64_t)c.num_sms);
     KernelScope ks("perm_dispatch", c.stream);
     perm_rank_kernel<true><<<grid, kRankWarps * 32, 0, c.stream>>>(

@@ -39,3 +39,27 @@ def test_expert_backward_dx_over_an_input(over, counts, D, F, dtype):
         out.append((dx, dw1, dw2))
     assert abi.moe_check_device_status() == 0
     assert all(torch.equal(p, q) for p, q in zip(*out))
+
+
+@pytest.mark.parametrize("T,K,D", [(1, 1, 64), (128, 4, 512), (500, 1, 1024), (300, 3, 256)])
+def test_dispatch_rows_over_the_indices(T, K, D):
+    """moe_dispatch with row_of_slot over topk_idx, on both sides of the size up
+    to which ranking and row copies are one launch."""
+    E = 64
+    g = torch.Generator(device="cuda").manual_seed(T)
+    shp = abi.MoeShape.of(T, 1, K, D, E, 64)
+    x = torch.randn(T, D, generator=g, device="cuda").bfloat16()
+    top = torch.topk(torch.randn(T, E, generator=g, device="cuda"), K, dim=1)
+    prob = torch.softmax(top.values, 1).contiguous()
+    ws = torch.empty(abi.moe_workspace_size(shp), dtype=torch.uint8, device="cuda")
+    i32 = dict(dtype=torch.int32, device="cuda")
+    out = []
+    for shared in (False, True):
+        idx = top.indices.to(torch.int32).contiguous()
+        ros = idx.view(-1) if shared else torch.empty(T * K, **i32)
+        off, tor, pp = torch.empty(E + 1, **i32), torch.empty(T * K, **i32), torch.empty(T * K, device="cuda")
+        xp = torch.empty(T * K, D, dtype=torch.bfloat16, device="cuda")
+        abi.moe_dispatch(shp, x, idx, prob, off, ros, tor, xp, pp, ws)
+        out.append((off, ros, tor, xp, pp))
+    assert abi.moe_check_device_status() == 0
+    assert all(torch.equal(p, q) for p, q in zip(*out))
