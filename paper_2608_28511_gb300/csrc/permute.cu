@@ -231,7 +231,7 @@ static inline int row_parts(const Ctx& c, int64_t T, int K, int vpr) {
   return vpr >= 128 && T * K < (int64_t)c.num_sms * 16 ? 8 : 1;
 }
 // Token and part of this warp: the parts of a token are consecutive warps of one
-// block of 8.
+// block of 8, which then holds that token alone.
 struct WarpToken {
   int64_t t;
   int part;
@@ -452,7 +452,9 @@ __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const uint4* __restri
     }
     st_stream(dx + t * ldv + v, pack16<T>(acc));
   }
-  // the probability gradients last, off the path of the row loads
+  // the probability gradients last, off the path of the row loads; dprob may lie
+  // over row_of_slot, which all parts have used by then
+  if (P > 1) __syncthreads();
   if (part == 0 && lane < K) dprob[t * K + lane] = __ldg(dprob_perm + row_of_slot[t * K + lane]);
 }
 
@@ -554,7 +556,6 @@ __global__ void __launch_bounds__(256, KM <= 8 ? 3 : 1) dispatch_route_bwd_kerne
     }
     st_stream(dx + t * vpr + v, pack16<T>(acc));
   }
-  if (part == 0 && lane < K) dprob[t * K + lane] = my_dp;
   for (int e0 = part * 32; e0 < E; e0 += 32 * P) {
     const int e = e0 + lane;
     float val = 0.f;
@@ -566,6 +567,9 @@ __global__ void __launch_bounds__(256, KM <= 8 ? 3 : 1) dispatch_route_bwd_kerne
       if (dz16) dz16[t * E + e] = __float2bfloat16_rn(val);
     }
   }
+  // dprob may lie over prob, which all parts have used by then
+  if (P > 1) __syncthreads();
+  if (part == 0 && lane < K) dprob[t * K + lane] = my_dp;
 }
 
 cudaError_t launch_dispatch_route_bwd(const Ctx& c, DType dt, const void* dx_perm, const float* dprob_perm,

@@ -63,3 +63,29 @@ def test_dispatch_rows_over_the_indices(T, K, D):
         out.append((off, ros, tor, xp, pp))
     assert abi.moe_check_device_status() == 0
     assert all(torch.equal(p, q) for p, q in zip(*out))
+
+
+@pytest.mark.parametrize("T,K,D", [(1, 1, 1024), (300, 8, 2048), (150, 16, 1024), (900, 2, 2560), (700, 4, 256)])
+def test_probability_gradient_over_the_probabilities(T, K, D):
+    """The dispatch backwards with dtopk_prob over topk_prob, and over row_of_slot,
+    with a token's row moved by one warp or by eight."""
+    E = 64
+    g = torch.Generator(device="cuda").manual_seed(T)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")  # noqa: E731
+    shp = abi.MoeShape.of(T, 1, K, D, E, 64)
+    x, w, dxp, dpp = rnd(T, D).bfloat16(), rnd(E, D).bfloat16(), rnd(T * K, D).bfloat16(), rnd(T * K)
+    top = torch.topk(rnd(T, E), K, dim=1)
+    idx, p0 = top.indices.to(torch.int32).contiguous(), torch.softmax(top.values, 1).contiguous()
+    ros0 = torch.randperm(T * K, generator=g, device="cuda").to(torch.int32)
+    ws = torch.empty(abi.moe_workspace_size(shp), dtype=torch.uint8, device="cuda")
+    out = []
+    for shared in (False, True):
+        prob, ros = p0.clone(), ros0.clone()
+        dprob = prob if shared else torch.empty_like(prob)
+        dx, dz, dwr = torch.empty_like(x), torch.empty(T, E, device="cuda"), torch.empty(E, D, device="cuda")
+        abi.moe_dispatch_route_bwd(shp, dxp, dpp, ros, x, w, idx, prob, dx, dprob, dz, dwr, ws)
+        dx2, dp2 = torch.empty_like(x), ros.view(torch.float32) if shared else torch.empty(T * K, device="cuda")
+        abi.moe_dispatch_bwd(shp, dxp, dpp, ros, dx2, dp2)
+        out.append((dx, dprob, dz, dwr, dx2, dp2))
+    assert abi.moe_check_device_status() == 0
+    assert all(torch.equal(p, q) for p, q in zip(*out))
