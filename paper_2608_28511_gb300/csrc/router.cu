@@ -20,17 +20,17 @@ __global__ void __launch_bounds__(256) topk_kernel(const float* __restrict__ log
   const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (t >= T) return;  // the whole warp
   const float* row = logits + t * E;
-  float key[V];
+  float z[V];
 #pragma unroll
-  for (int v = 0; v < V; ++v)
-    key[v] = v * 32 + lane < E ? sel::key_of(__ldg(row + v * 32 + lane)) : __uint_as_float(sel::kAbsent);
-  float mk, best;
-  int me;
-  sel::warp_topk<V>(key, E, K, lane, slots[threadIdx.x >> 5], [&] { return row; }, &mk, &me, &best);
-  const float w = lane < K ? expf(mk - best) : 0.f;
+  for (int v = 0; v < V; ++v) z[v] = v * 32 + lane < E ? __ldg(row + v * 32 + lane) : 0.f;
+  uint2* slot = slots[threadIdx.x >> 5];
+  sel::warp_topk<V>([&](int v) { return v * 32 + lane < E ? sel::key_of(z[v]) : __uint_as_float(sel::kAbsent); }, K,
+                    lane, slot);
+  const float best = __uint_as_float(slot[0].x);
+  const float w = lane < K ? expf(__uint_as_float(slot[lane].x) - best) : 0.f;
   const float inv = 1.0f / sel::sum_chosen(w, K);
   if (lane < K) {
-    idx[t * K + lane] = me;
+    idx[t * K + lane] = (int)(slot[lane].y & 255u);
     prob[t * K + lane] = w * inv;
   }
 }

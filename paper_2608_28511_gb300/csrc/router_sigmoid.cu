@@ -35,13 +35,14 @@ constexpr int kSelWarps = 16;
 // Bound by each warp's chain of tokens: at T = 8192, E = 64, K = 6 it takes
 // 10.4 us, 13.6 with eight warps; staging 64 rows in shared memory and selecting
 // with four threads per token took 14.3.
+// Two blocks per SM need 64 registers a thread (V = 8 takes 74 by itself): T = 16384,
+// E = 256, K = 8 33 -> 27 us.
 template <int V>
-__global__ void __launch_bounds__(32 * kSelWarps) select_sigmoid_kernel(
+__global__ void __launch_bounds__(32 * kSelWarps, V == 8 ? 2 : 1) select_sigmoid_kernel(
     const float* __restrict__ logits, const float* __restrict__ bias, int64_t S, int E, int K, int tpb, int nch,
     int32_t* __restrict__ idx, float* __restrict__ prob, float* __restrict__ psum, int32_t* __restrict__ pcnt,
     uint32_t* __restrict__ ticket, float* __restrict__ keys) {
   __shared__ float wsum[kSelWarps][V * 32];
-  __shared__ float tie_row[kSelWarps][V * 32];
   __shared__ uint2 slots[kSelWarps][kMaxK];
   __shared__ int cnt[V * 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ch = blockIdx.x, g = blockIdx.y;
@@ -66,34 +67,25 @@ __global__ void __launch_bounds__(32 * kSelWarps) select_sigmoid_kernel(
   for (int q = q0; q < q1; ++q) {
     const int64_t t = t0 + q;
     float s[V];
-    float key[V];
     float ssum = 0.f;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const bool in = v * 32 + lane < E;
       s[v] = in ? sigmoidf_(z[v]) : 0.f;
-      const float k = __fadd_rn(s[v], b[v]);
-      key[v] = in ? sel::key_of(k) : __uint_as_float(sel::kAbsent);
-      if (keys && in) keys[t * E + v * 32 + lane] = k;
+      if (keys && in) keys[t * E + v * 32 + lane] = __fadd_rn(s[v], b[v]);
       ssum += s[v];
     }
     if (q + 1 < q1) fetch(q + 1);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ssum += __shfl_xor_sync(0xffffffffu, ssum, o);
-    float mk, best;
-    int me;
+    uint2* slot = slots[warp];
     sel::warp_topk<V>(
-        key, E, K, lane, slots[warp],
-        [&] {
-          // rare: the keys again, where topk_with_ties can read them
-          __syncwarp();
-#pragma unroll
-          for (int v = 0; v < V; ++v) tie_row[warp][v * 32 + lane] = __fadd_rn(s[v], b[v]);
-          __syncwarp();
-          return (const float*)tie_row[warp];
+        [&](int v) {
+          return v * 32 + lane < E ? sel::key_of(__fadd_rn(s[v], b[v])) : __uint_as_float(sel::kAbsent);
         },
-        &mk, &me, &best);
+        K, lane, slot);
     // lane k: the k-th chosen expert's score, from the lane that holds it
+    const int me = lane < K ? (int)(slot[lane].y & 255u) : 0;
     float sk = 0.f;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -106,6 +98,7 @@ __global__ void __launch_bounds__(32 * kSelWarps) select_sigmoid_kernel(
       prob[t * K + lane] = sk * ginv;
       atomicAdd(cnt + me, 1);
     }
+    __syncwarp();  // the slots are read before the next token's rounds write them
     const float inv = __frcp_rn(ssum);
 #pragma unroll
     for (int v = 0; v < V; ++v) acc[v] += s[v] * inv;

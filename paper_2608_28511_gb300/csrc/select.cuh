@@ -5,15 +5,19 @@
 // with one warp reduction (redux.sync.max.f32), and the lane whose head it is
 // records it and drops it.
 //
-// Rounds assume that all chosen keys differ, and the end checks it: one head
-// taken per round, no two taken keys equal, none left equal to the last one.
-// Otherwise the token is chosen again by rounds that resolve equal keys to the
-// lower expert.  -0 ties with +0 and NaN keys count as -inf.
+// Rounds assume that all chosen keys differ.  The first one shows whether the
+// best key is in several lanes, and the end checks the rest: one head taken per
+// round, no two taken keys equal, none left equal to the last one.  Otherwise the
+// token is chosen again by rounds that take every key equal to the largest one
+// left, in the order of the experts.  -0 ties with +0 and NaN keys count as -inf.
 //
 // Bound by the compare / select pipe, then by the chain of K reductions.  At
 // T = 30011, E = 128, K = 8 the top-K kernel takes 14.3 us; four threads per
 // token with sorted insertion lists took 29.7, rounds that track each owner's
-// expert by vote and shuffle 18.3.
+// expert by vote and shuffle 18.3.  Equal keys (logits of a router that starts at
+// zero, scores that saturate), T = 16384, E = 256, K = 8, inputs in L2: all equal
+// 8.9 us, one equal pair 15.2, none 9.2; with all K rounds first and then rounds
+// that take one key each 20.5, 20.5 and 9.3.
 #pragma once
 
 #include <math_constants.h>
@@ -34,7 +38,7 @@ __device__ __forceinline__ float warp_max(float v) {
   return m;
 }
 
-// Lists of 32 experts that E takes, and a bound on K, as compile-time sizes.
+// Lists of 32 experts that E takes, as a compile-time size.
 inline int lists_of(int E) { return E <= 32 ? 1 : E <= 64 ? 2 : E <= 128 ? 4 : 8; }
 
 // Comparators that sort V keys (Batcher's odd-even merge sort).
@@ -63,47 +67,22 @@ __device__ __forceinline__ void sort_lists(float (&key)[V], uint32_t (&id)[V]) {
   }
 }
 
-// The rounds for keys that may be equal: ties go to the lower expert.
-template <int V>
-__device__ __noinline__ uint2 topk_with_ties(const float* row, int E, int K, int lane) {
-  // row: the warp's keys in shared or global memory, expert by expert
-  float key[V];
-#pragma unroll
-  for (int v = 0; v < V; ++v)
-    key[v] = v * 32 + lane < E ? key_of(row[v * 32 + lane]) : __uint_as_float(kAbsent);
-  uint2 r = make_uint2(0u, 0u);
-  for (int k = 0; k < K; ++k) {
-    float h = key[0];
-    unsigned he = (unsigned)lane;
-#pragma unroll
-    for (int v = 1; v < V; ++v) {
-      if (key[v] > h || h != h) {  // strictly larger: the lower expert keeps a tie
-        h = key[v];
-        he = (unsigned)(v * 32 + lane);
-      }
-    }
-    const float m = warp_max(h);
-    const unsigned e = __reduce_min_sync(0xffffffffu, h == m ? he : 0xffffffffu);
-    if (lane == k) r = make_uint2(__float_as_uint(m), e);
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-      if (e == (unsigned)(v * 32 + lane)) key[v] = __uint_as_float(kAbsent);
-  }
-  return r;
-}
-
-// The K <= 16 best of a token's E keys: key[v] = key_of(expert 32 v + lane's),
-// absent where there is none.  slot: 16 entries of shared memory of this warp's
-// own; row(): the same keys in memory (read only where keys are equal).  Lane
-// k < K returns the k-th best's key and expert, the other lanes 0 and 0; *best
-// is the best key, in every lane.  The whole warp calls.
-template <int V, typename Row>
-__device__ __forceinline__ void warp_topk(float (&key)[V], int E, int K, int lane, uint2* slot, Row row,
-                                          float* my_key, int* my_e, float* best) {
+// The K <= 16 best of a token's E keys: lane l holds the keys of experts l,
+// l + 32, ..., keys(v) being key_of(expert 32 v + l's), absent where there is
+// none (called again where keys are equal).  slot: 16 entries of shared memory of
+// this warp's own, of which 0 .. K - 1 receive the best ones' keys and (in the low
+// byte) experts, best first.  The whole warp calls, and calls __syncwarp() between
+// reading the slots and the next token.
+template <int V, typename Keys>
+__device__ __forceinline__ void warp_topk(Keys keys, int K, int lane, uint2* slot) {
   const float absent = __uint_as_float(kAbsent);
+  float key[V];
   uint32_t id[V];
 #pragma unroll
-  for (int v = 0; v < V; ++v) id[v] = (uint32_t)(v * 32 + lane);
+  for (int v = 0; v < V; ++v) {
+    key[v] = keys(v);
+    id[v] = (uint32_t)(v * 32 + lane);
+  }
   sort_lists<V>(key, id);
   // the list's experts, a byte each, first to last: dropping the head is a shift
   uint32_t lo = 0, hi = 0;
@@ -112,38 +91,62 @@ __device__ __forceinline__ void warp_topk(float (&key)[V], int E, int K, int lan
     if (v < 4) lo |= id[v] << (8 * v);
     else hi |= id[v] << (8 * (v - 4));
   }
-  int taken = 0;
-  float m = 0.f;
+  float m = warp_max(key[0]);
+  const unsigned heads = __ballot_sync(0xffffffffu, key[0] == m);
+  bool ties = (heads & (heads - 1u)) != 0u;
+  if (!ties) {
+    int taken = 0;
 #pragma unroll 2
-  for (int k = 0; k < K; ++k) {
-    m = warp_max(key[0]);
-    if (key[0] == m) {
-      slot[k] = make_uint2(__float_as_uint(m), lo);
-      ++taken;
+    for (int k = 0;;) {
+      if (key[0] == m) {
+        slot[k] = make_uint2(__float_as_uint(m), lo);
+        ++taken;
 #pragma unroll
-      for (int v = 0; v + 1 < V; ++v) key[v] = key[v + 1];
-      key[V - 1] = absent;
-      if (V > 4) {
-        lo = __funnelshift_r(lo, hi, 8);
-        hi >>= 8;
-      } else {
-        lo >>= 8;
+        for (int v = 0; v + 1 < V; ++v) key[v] = key[v + 1];
+        key[V - 1] = absent;
+        if (V > 4) {
+          lo = __funnelshift_r(lo, hi, 8);
+          hi >>= 8;
+        } else {
+          lo >>= 8;
+        }
+      }
+      if (++k == K) break;
+      m = warp_max(key[0]);
+    }
+    __syncwarp();
+    const float mine = lane < K ? __uint_as_float(slot[lane].x) : 0.f;
+    const float next = __shfl_down_sync(0xffffffffu, mine, 1);
+    // m is NaN if the keys ran out, which takes an earlier round that took several
+    const bool tie = key[0] == m || m != m || (lane + 1 < K && mine == next);
+    ties = __reduce_add_sync(0xffffffffu, (unsigned)taken) != (unsigned)K || __any_sync(0xffffffffu, tie);
+  }
+  if (ties) {
+    // keys that may be equal: each round takes every key that equals the largest
+    // one left, in the order of the experts, so equal keys cost one round together
+#pragma unroll
+    for (int v = 0; v < V; ++v) key[v] = keys(v);
+    __syncwarp();
+    int got = 0;
+    for (int k = 0; k < K && got < K; ++k) {
+      float h = key[0];
+#pragma unroll
+      for (int v = 1; v < V; ++v) h = fmaxf(h, key[v]);
+      m = warp_max(h);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const bool eq = key[v] == m;
+        const unsigned b = __ballot_sync(0xffffffffu, eq);
+        if (eq) {
+          const int at = got + __popc(b & ((1u << lane) - 1u));
+          if (at < K) slot[at] = make_uint2(__float_as_uint(m), (unsigned)(v * 32 + lane));
+          key[v] = absent;
+        }
+        got += __popc(b);
       }
     }
+    __syncwarp();
   }
-  __syncwarp();
-  uint2 r = make_uint2(0u, 0u);
-  if (lane < K) r = slot[lane];
-  r.y &= 255u;
-  const float mine = __uint_as_float(r.x), next = __shfl_down_sync(0xffffffffu, mine, 1);
-  // m is NaN if the keys ran out, which takes an earlier round that took several
-  const bool tie = key[0] == m || m != m || (lane + 1 < K && mine == next);
-  if (__reduce_add_sync(0xffffffffu, (unsigned)taken) != (unsigned)K || __any_sync(0xffffffffu, tie))
-    r = topk_with_ties<V>(row(), E, K, lane);
-  *my_key = __uint_as_float(r.x);
-  *my_e = (int)r.y;
-  *best = __shfl_sync(0xffffffffu, *my_key, 0);
-  __syncwarp();  // the slots are read before the next token's rounds write them
 }
 
 // The sum of the values of lanes 0 .. K - 1, added in that order (best expert

@@ -64,3 +64,38 @@ def test_probabilities_are_summed_best_first(K):
     abi.moe_topk_sigmoid(shp, z.cuda(), None, 1e-4, None, idx, prob, f, loss, ws)
     assert torch.equal(idx[:, 0].cpu().long(), best) and bool((prob[:, 0] == 1.0).all())
     assert abi.moe_check_device_status() == 0
+
+
+@pytest.mark.parametrize("E,K", [(3, 3), (32, 16), (40, 8), (64, 5), (128, 16), (200, 8), (256, 16)])
+def test_equal_keys_in_every_place(E, K):
+    """Pairs and runs of equal keys at each rank up to past the last chosen one, in
+    one lane (experts 32 apart) and across lanes, and rows that hold few distinct
+    keys: the lower expert comes first."""
+    g = torch.Generator().manual_seed(E + K)
+    rows = []
+    for r in range(min(K + 1, E - 1)):
+        for run in (2, 3, 40):
+            for shift in (1, 32):
+                z = torch.randn(E, generator=g).sort(descending=True).values
+                z[r : r + run] = z[r].clone()                      # ranks r .. r + run - 1 are equal
+                order = torch.randperm(E, generator=g)
+                place = torch.empty(E)
+                if shift == 32:                                    # ... and lie 32 experts apart
+                    order = torch.arange(E).view(-1, 1) if E <= 32 else torch.argsort(torch.arange(E) % 32, stable=True)
+                    order = order.reshape(-1).roll(int(torch.randint(E, (1,), generator=g)))
+                place[order] = z
+                rows.append(place)
+    for n in (1, 2, 3):
+        rows += list(torch.randint(0, n, (20, E), generator=g).float())
+    z = torch.stack(rows)
+    T = z.shape[0]
+    idx, prob = torch.empty(T, K, dtype=torch.int32, device="cuda"), torch.empty(T, K, device="cuda")
+    shp = abi.MoeShape.of(T, 1, K, 64, E, 64)
+    ref = np.argsort(-z.numpy(), axis=1, kind="stable")[:, :K]
+    abi.moe_topk(shp, z.cuda(), idx, prob)
+    assert (idx.cpu().numpy() == ref).all()
+    keys, f, loss = torch.empty(T, E, device="cuda"), torch.empty(1, E, device="cuda"), torch.empty(4, device="cuda")
+    ws = torch.empty(abi.moe_workspace_size(shp), dtype=torch.uint8, device="cuda")
+    abi.moe_topk_sigmoid(shp, z.cuda(), None, 1e-4, keys, idx, prob, f, loss, ws)
+    ref = np.argsort(-keys.cpu().numpy(), axis=1, kind="stable")[:, :K]
+    assert (idx.cpu().numpy() == ref).all() and abi.moe_check_device_status() == 0
