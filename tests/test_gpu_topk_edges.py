@@ -99,3 +99,31 @@ def test_equal_keys_in_every_place(E, K):
     abi.moe_topk_sigmoid(shp, z.cuda(), None, 1e-4, keys, idx, prob, f, loss, ws)
     ref = np.argsort(-keys.cpu().numpy(), axis=1, kind="stable")[:, :K]
     assert (idx.cpu().numpy() == ref).all() and abi.moe_check_device_status() == 0
+
+
+@pytest.mark.parametrize("E", [5, 16, 20, 64, 130])
+@pytest.mark.parametrize("S,GBS", [(1, 3), (4, 5), (15, 2), (17, 2), (33, 1), (63, 2), (65, 3), (100, 1)])
+def test_sigmoid_statistics_of_short_sequences(S, GBS, E):
+    """Choice counts and the balance loss where a sequence does not give every warp
+    of a block the same number of tokens: f exactly from the choices, the loss
+    against float64 (a mean of T fp32 quotients: within 1e-6)."""
+    K, T = min(E, 3), S * GBS
+    g = torch.Generator().manual_seed(S * E)
+    z, b = torch.randn(T, E, generator=g), torch.randn(E, generator=g) * 0.05
+    shp = abi.MoeShape.of(S, GBS, K, 64, E, 64)
+    idx, prob = torch.empty(T, K, dtype=torch.int32, device="cuda"), torch.empty(T, K, device="cuda")
+    f, loss = torch.empty(GBS, E, device="cuda"), torch.empty(4, device="cuda")
+    keys = torch.empty(T, E, device="cuda")
+    ws = torch.empty(abi.moe_workspace_size(shp), dtype=torch.uint8, device="cuda")
+    abi.moe_topk_sigmoid(shp, z.cuda(), b.cuda(), 0.5, keys, idx, prob, f, loss, ws)
+    assert abi.moe_check_device_status() == 0
+    i = idx.cpu().long()
+    assert (i.numpy() == np.argsort(-keys.cpu().numpy(), axis=1, kind="stable")[:, :K]).all()
+    s = torch.sigmoid(z.double())
+    cnt = torch.zeros(T, E, dtype=torch.float64).scatter_(1, i, 1.0).view(GBS, S, E).sum(1)
+    assert float((f.cpu().double() - cnt * E / (K * S)).abs().max()) <= 1e-6 * E
+    sel = s.gather(1, i)
+    assert float((prob.cpu().double() - sel / sel.sum(1, keepdim=True)).abs().max()) <= 1e-6
+    P = (s / s.sum(1, keepdim=True)).view(GBS, S, E).mean(1)
+    want = 0.5 / GBS * float((cnt * E / (K * S) * P).sum())
+    assert abs(float(loss[0]) - want) <= 2e-6 * abs(want)
