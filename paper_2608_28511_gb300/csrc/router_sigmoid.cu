@@ -36,10 +36,11 @@ constexpr int kSelWarps = 16;
 // Bound by each warp's chain of tokens: at T = 8192, E = 64, K = 6 it takes
 // 10.4 us, 13.6 with eight warps; staging 64 rows in shared memory and selecting
 // with four threads per token took 14.3.
-// Two blocks per SM need 64 registers a thread (V = 8 takes 74 by itself): T = 16384,
-// E = 256, K = 8 33 -> 27 us.
+// At least two blocks per SM (64 registers a thread; V = 8 takes 74 by itself:
+// T = 16384, E = 256, K = 8 33 -> 27 us), three for short lists (40 registers, not
+// 50).
 template <int V>
-__global__ void __launch_bounds__(32 * kSelWarps, V == 8 ? 2 : 1) select_sigmoid_kernel(
+__global__ void __launch_bounds__(32 * kSelWarps, V <= 2 ? 3 : 2) select_sigmoid_kernel(
     const float* __restrict__ logits, const float* __restrict__ bias, int64_t S, int E, int K, int tpb, int nch,
     int32_t* __restrict__ idx, float* __restrict__ prob, float* __restrict__ psum, int32_t* __restrict__ pcnt,
     uint32_t* __restrict__ ticket, float* __restrict__ keys) {
