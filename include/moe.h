@@ -96,7 +96,7 @@ int moe_workspace_size(const moe_shape_t* shape, size_t* bytes);
 int moe_route(const moe_shape_t* shape, const void* x, const void* w_router, const float* bias,
               float* logits, int32_t* topk_idx, float* topk_prob, void* ws, size_t ws_bytes, void* stream);
 
-/* Top-K of given fp32 logits [T, E] (one warp per token): the K largest
+/* Top-K of given fp32 logits [T, E]: the K largest
  * logits (ties to the lower expert index), ordered by descending logit, and
  * renormalised probabilities p_k = exp(z_k - z_max) / sum over the K chosen
  * (equal to softmax over all E restricted to the chosen set). */

@@ -8,43 +8,49 @@
 
 namespace moe {
 
-// One warp per token (select.cuh): the K largest logits, ties to the lower
-// expert index (reading R2), NaN as -inf, ordered by descending logit.  The
-// probabilities are exp(z_k - z_max) normalised over the K chosen logits,
+// One warp or a few lanes per token (select.cuh): the K largest logits, ties to
+// the lower expert index (reading R2), NaN as -inf, ordered by descending logit.
+// The probabilities are exp(z_k - z_max) normalised over the K chosen logits,
 // which equals the full softmax renormalised over the chosen set (reading R1).
-template <int V>
+template <int V, int G>
 __global__ void __launch_bounds__(256) topk_kernel(const float* __restrict__ logits, int64_t T, int E, int K,
                                                    int32_t* __restrict__ idx, float* __restrict__ prob) {
-  __shared__ uint2 slots[8][kMaxK];
-  const int lane = threadIdx.x & 31;
-  const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (t >= T) return;  // the whole warp
+  constexpr int TW = 32 / G, P = sel::kPerLane<V, G>;
+  __shared__ uint2 slots[8][TW][kMaxK];
+  const int warp = threadIdx.x >> 5, sub = (threadIdx.x & 31) / G, l = threadIdx.x % G;
+  const int64_t t0 = ((int64_t)blockIdx.x * 8 + warp) * TW, t = t0 + sub;
+  if (t0 >= T) return;  // the whole warp
   const float* row = logits + t * E;
   float z[V];
 #pragma unroll
-  for (int v = 0; v < V; ++v) z[v] = v * 32 + lane < E ? __ldg(row + v * 32 + lane) : 0.f;
-  uint2* slot = slots[threadIdx.x >> 5];
-  sel::warp_topk<V>([&](int v) { return v * 32 + lane < E ? sel::key_of(z[v]) : __uint_as_float(sel::kAbsent); }, K,
-                    lane, slot);
+  for (int v = 0; v < V; ++v) z[v] = t < T && v * G + l < E ? __ldg(row + v * G + l) : 0.f;
+  const uint2* slot = slots[warp][sub];
+  sel::token_topk<V, G>(
+      [&](int v) { return v * G + l < E ? sel::key_of(z[v]) : __uint_as_float(sel::kAbsent); }, E, K, l,
+      slots[warp][sub]);
   const float best = __uint_as_float(slot[0].x);
-  const float w = lane < K ? expf(__uint_as_float(slot[lane].x) - best) : 0.f;
-  const float inv = 1.0f / sel::sum_chosen(w, K);
-  if (lane < K) {
-    idx[t * K + lane] = (int)(slot[lane].y & 255u);
-    prob[t * K + lane] = w * inv;
+  float w[P];
+#pragma unroll
+  for (int p = 0; p < P; ++p) w[p] = p * G + l < K ? expf(__uint_as_float(slot[p * G + l].x) - best) : 0.f;
+  const float inv = 1.0f / sel::sum_chosen<P, G>(w, K);
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const int k = p * G + l;
+    if (k < K && t < T) {
+      idx[t * K + k] = (int)(slot[k].y & 255u);
+      prob[t * K + k] = w[p] * inv;
+    }
   }
 }
 
 cudaError_t launch_topk(const Ctx& c, const float* logits, int64_t T, int E, int K, int32_t* idx, float* prob) {
   if (T == 0) return cudaSuccess;
-  const unsigned grid = (unsigned)((T + 7) / 8);
   KernelScope ks("topk", c.stream);
-  switch (sel::lists_of(E)) {
-    case 1: topk_kernel<1><<<grid, 256, 0, c.stream>>>(logits, T, E, K, idx, prob); break;
-    case 2: topk_kernel<2><<<grid, 256, 0, c.stream>>>(logits, T, E, K, idx, prob); break;
-    case 4: topk_kernel<4><<<grid, 256, 0, c.stream>>>(logits, T, E, K, idx, prob); break;
-    default: topk_kernel<8><<<grid, 256, 0, c.stream>>>(logits, T, E, K, idx, prob); break;
-  }
+  sel::for_experts(E, [&](auto v, auto g) {
+    constexpr int G = decltype(g)::value, per = 8 * 32 / G;  // tokens per block
+    topk_kernel<decltype(v)::value, G>
+        <<<(unsigned)((T + per - 1) / per), 256, 0, c.stream>>>(logits, T, E, K, idx, prob);
+  });
   return cudaGetLastError();
 }
 

@@ -27,27 +27,32 @@ constexpr int kSelWarps = 16;
 
 // Block (chunk ch of sequence g): kSelWarps warps, each with an equal run of
 // the chunk's tokens (a short sequence has fewer, down to one per warp: 2048
-// sequences of 4 tokens, E = 64, K = 6 46 -> 25 us).  Per token the warp forms the scores s = sigmoid(z) in
-// registers, chooses the K experts by s + b (select.cuh), writes idx and the
-// gate values s_k / sum over the chosen of s, and adds the normalised scores of
-// its experts (in token order) and, in shared memory, the choice counts.  The
-// warps' sums are then added in order: one partial per (sequence, chunk).
-// With `keys` the warp also writes every selection key s + b it compared.
+// sequences of 4 tokens, E = 64, K = 6 46 -> 25 us).  Per token a warp, or for up
+// to 32 experts a group of G lanes, forms the scores s = sigmoid(z) in registers,
+// chooses the K experts by s + b (select.cuh), writes idx and the gate values
+// s_k / sum over the chosen of s, and adds the normalised scores of its experts
+// (in token order) and, in shared memory, the choice counts.  The sums are then
+// added in order: one partial per (sequence, chunk).  With `keys` every selection
+// key s + b that was compared is written too.
 // Bound by each warp's chain of tokens: at T = 8192, E = 64, K = 6 it takes
 // 10.4 us, 13.6 with eight warps; staging 64 rows in shared memory and selecting
-// with four threads per token took 14.3.
+// with four threads per token took 14.3.  E = 8, K = 2, T = 16384 with the balance
+// statistics: 11.2 us with a warp per token, 8.3 with groups.
 // At least two blocks per SM (64 registers a thread; V = 8 takes 74 by itself:
 // T = 16384, E = 256, K = 8 33 -> 27 us), three for short lists (40 registers, not
 // 50).
-template <int V>
+template <int V, int G>
 __global__ void __launch_bounds__(32 * kSelWarps, V <= 2 ? 3 : 2) select_sigmoid_kernel(
     const float* __restrict__ logits, const float* __restrict__ bias, int64_t S, int E, int K, int tpb, int nch,
     int32_t* __restrict__ idx, float* __restrict__ prob, float* __restrict__ psum, int32_t* __restrict__ pcnt,
     uint32_t* __restrict__ ticket, float* __restrict__ keys) {
+  constexpr int TW = 32 / G;  // tokens of a warp at once
+  constexpr int P = sel::kPerLane<V, G>;
   __shared__ float wsum[kSelWarps][V * 32];
-  __shared__ uint2 slots[kSelWarps][kMaxK];
+  __shared__ uint2 slots[kSelWarps][TW][kMaxK];
   __shared__ int cnt[V * 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ch = blockIdx.x, g = blockIdx.y;
+  const int sub = lane / G, l = lane % G;
   const int64_t t0 = (int64_t)g * S + (int64_t)ch * tpb;
   const int n = (int)min((int64_t)tpb, S - (int64_t)ch * tpb);
   for (int e = tid; e < V * 32; e += 32 * kSelWarps) cnt[e] = 0;
@@ -56,52 +61,62 @@ __global__ void __launch_bounds__(32 * kSelWarps, V <= 2 ? 3 : 2) select_sigmoid
   float b[V], acc[V], z[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    b[v] = bias && v * 32 + lane < E ? __ldg(bias + v * 32 + lane) : 0.f;
+    b[v] = bias && v * G + l < E ? __ldg(bias + v * G + l) : 0.f;
     acc[v] = 0.f;
   }
   auto fetch = [&](int q) {
 #pragma unroll
     for (int v = 0; v < V; ++v)
-      z[v] = q < n && v * 32 + lane < E ? __ldg(logits + (t0 + q) * E + v * 32 + lane) : 0.f;
+      z[v] = q < n && v * G + l < E ? __ldg(logits + (t0 + q) * E + v * G + l) : 0.f;
   };
-  const int per = (n + kSelWarps - 1) / kSelWarps, q0 = warp * per, q1 = min(n, q0 + per);
-  fetch(q0);
-  for (int q = q0; q < q1; ++q) {
-    const int64_t t = t0 + q;
+  const int per = ((n + kSelWarps - 1) / kSelWarps + TW - 1) / TW * TW, q0 = warp * per, q1 = min(n, q0 + per);
+  fetch(q0 + sub);
+  for (int q = q0; q < q1; q += TW) {
+    const int64_t t = t0 + q + sub;
+    const bool live = TW == 1 || q + sub < q1;
     float s[V];
     float ssum = 0.f;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-      const bool in = v * 32 + lane < E;
+      const bool in = v * G + l < E;
       s[v] = in ? sigmoidf_(z[v]) : 0.f;
-      if (keys && in) keys[t * E + v * 32 + lane] = __fadd_rn(s[v], b[v]);
+      if (keys && in && live) keys[t * E + v * G + l] = __fadd_rn(s[v], b[v]);
       ssum += s[v];
     }
-    if (q + 1 < q1) fetch(q + 1);
+    if (q + TW < q1) fetch(q + TW + sub);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ssum += __shfl_xor_sync(0xffffffffu, ssum, o);
-    uint2* slot = slots[warp];
-    sel::warp_topk<V>(
+    for (int o = G / 2; o > 0; o >>= 1) ssum += __shfl_xor_sync(0xffffffffu, ssum, o);
+    const uint2* slot = slots[warp][sub];
+    sel::token_topk<V, G>(
         [&](int v) {
-          return v * 32 + lane < E ? sel::key_of(__fadd_rn(s[v], b[v])) : __uint_as_float(sel::kAbsent);
+          return v * G + l < E ? sel::key_of(__fadd_rn(s[v], b[v])) : __uint_as_float(sel::kAbsent);
         },
-        K, lane, slot);
-    // lane k: the k-th chosen expert's score, from the lane that holds it
-    const int me = lane < K ? (int)(slot[lane].y & 255u) : 0;
-    float sk = 0.f;
+        E, K, l, slots[warp][sub]);
+    // the chosen experts' scores, from the lanes that hold them
+    int me[P];
+    float sk[P];
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const float sv = __shfl_sync(0xffffffffu, s[v], me & 31);
-      if (me >> 5 == v && lane < K) sk = sv;
+    for (int p = 0; p < P; ++p) {
+      me[p] = p * G + l < K ? (int)(slot[p * G + l].y & 255u) : 0;
+      sk[p] = 0.f;
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const float sv = __shfl_sync(0xffffffffu, s[v], me[p] % G, G);
+        if (me[p] / G == v && p * G + l < K) sk[p] = sv;
+      }
     }
-    const float ginv = __frcp_rn(sel::sum_chosen(sk, K));
-    if (lane < K) {
-      idx[t * K + lane] = me;
-      prob[t * K + lane] = sk * ginv;
-      atomicAdd(cnt + me, 1);
+    const float ginv = __frcp_rn(sel::sum_chosen<P, G>(sk, K));
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      const int k = p * G + l;
+      if (k < K && live) {
+        idx[t * K + k] = me[p];
+        prob[t * K + k] = sk[p] * ginv;
+        atomicAdd(cnt + me[p], 1);
+      }
     }
     __syncwarp();  // the slots are read before the next token's rounds write them
-    const float inv = __frcp_rn(ssum);
+    const float inv = live ? __frcp_rn(ssum) : 0.f;
 #pragma unroll
     for (int v = 0; v < V; ++v) acc[v] += s[v] * inv;
   }
@@ -112,7 +127,9 @@ __global__ void __launch_bounds__(32 * kSelWarps, V <= 2 ? 3 : 2) select_sigmoid
   for (int e = tid; e < E; e += 32 * kSelWarps) {
     float sum = 0.f;
 #pragma unroll
-    for (int w = 0; w < kSelWarps; ++w) sum += wsum[w][e];
+    for (int w = 0; w < kSelWarps; ++w)
+#pragma unroll
+      for (int u = 0; u < TW; ++u) sum += wsum[w][e / G * 32 + u * G + e % G];
     psum[o + e] = sum;
     pcnt[o + e] = cnt[e];
   }
@@ -284,16 +301,11 @@ cudaError_t launch_route_sigmoid_select(const Ctx& c, const float* logits, const
   {
     dim3 grid((unsigned)nch, (unsigned)GBS);
     KernelScope ks("select_sigmoid", c.stream);
-#define MOE_SELECT_SIGMOID(V)                                                                                     \
-  select_sigmoid_kernel<V><<<grid, 32 * kSelWarps, 0, c.stream>>>(logits, bias, S, E, K, tpb, (int)nch, idx, prob, psum, pcnt, \
-                                                       ticket, keys)
-    switch (sel::lists_of(E)) {
-      case 1: MOE_SELECT_SIGMOID(1); break;
-      case 2: MOE_SELECT_SIGMOID(2); break;
-      case 4: MOE_SELECT_SIGMOID(4); break;
-      default: MOE_SELECT_SIGMOID(8); break;
-    }
-#undef MOE_SELECT_SIGMOID
+    sel::for_experts(E, [&](auto v, auto gl) {
+      select_sigmoid_kernel<decltype(v)::value, decltype(gl)::value>
+          <<<grid, 32 * kSelWarps, 0, c.stream>>>(logits, bias, S, E, K, tpb, (int)nch, idx, prob, psum, pcnt, ticket,
+                                                  keys);
+    });
   }
   cudaError_t st = cudaGetLastError();
   if (st != cudaSuccess) return st;

@@ -1,9 +1,10 @@
 // Top-K selection over the E experts of each token, shared by the softmax
 // router (keys = logits) and the sigmoid router (keys = sigmoid scores + expert
-// bias).  One warp per token: lane l holds experts l, l + 32, ... as a short
-// list sorted in registers; each of the K rounds takes the largest list head
-// with one warp reduction (redux.sync.max.f32), and the lane whose head it is
-// records it and drops it.
+// bias).  More than 32 experts: one warp per token; lane l holds experts l,
+// l + 32, ... as a short list sorted in registers; each of the K rounds takes the
+// largest list head with one warp reduction (redux.sync.max.f32), and the lane
+// whose head it is records it and drops it.  Up to 32 experts: four or eight
+// lanes per token (below).
 //
 // Rounds assume that all chosen keys differ.  The first one shows whether the
 // best key is in several lanes, and the end checks the rest: one head taken per
@@ -22,6 +23,8 @@
 
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace moe {
@@ -38,8 +41,17 @@ __device__ __forceinline__ float warp_max(float v) {
   return m;
 }
 
-// Lists of 32 experts that E takes, as a compile-time size.
-inline int lists_of(int E) { return E <= 32 ? 1 : E <= 64 ? 2 : E <= 128 ? 4 : 8; }
+// Runs f with the lists per lane (V) and lanes per token (G) for E experts.
+template <typename F>
+inline void for_experts(int E, F f) {
+  if (E <= 4) f(std::integral_constant<int, 1>(), std::integral_constant<int, 4>());
+  else if (E <= 8) f(std::integral_constant<int, 1>(), std::integral_constant<int, 8>());
+  else if (E <= 16) f(std::integral_constant<int, 2>(), std::integral_constant<int, 8>());
+  else if (E <= 32) f(std::integral_constant<int, 4>(), std::integral_constant<int, 8>());
+  else if (E <= 64) f(std::integral_constant<int, 2>(), std::integral_constant<int, 32>());
+  else if (E <= 128) f(std::integral_constant<int, 4>(), std::integral_constant<int, 32>());
+  else f(std::integral_constant<int, 8>(), std::integral_constant<int, 32>());
+}
 
 // Comparators that sort V keys (Batcher's odd-even merge sort).
 template <int V>
@@ -149,23 +161,113 @@ __device__ __forceinline__ void warp_topk(Keys keys, int K, int lane, uint2* slo
   }
 }
 
-// The sum of the values of lanes 0 .. K - 1, added in that order (best expert
-// first), in every lane: a probability is a function of its chosen keys alone,
-// not of how the lanes are paired.  Lanes K .. 15 pass 0.  The shuffles of a size
-// are in flight together; a loop to K takes them one by one (8192 sequences of
-// one token, E = 64, K = 6 90 us, now 77).
-template <int N>
-__device__ __forceinline__ float sum_first(float v) {
+// Tokens of up to 32 experts: G lanes each (32 / G tokens at once), lane l of a
+// group holding experts l, l + G, ...  A warp per token leaves lanes without an
+// expert and costs the same for 8 experts as for 32; T = 16384, K = 2, inputs in L2:
+// E = 8 3.7 -> 2.1 us, 16 3.7 -> 2.6, 32 3.7 -> 2.8 (four threads per token with
+// sorted lists 2.4, 2.7, 3.4); T = 65536, E = 8 10.3 -> 3.9.
+//
+// group_ranks: every lane counts the keys that come before each of its own, and
+// the chosen ones go to their places; the cost does not depend on K.
+template <int V, int G, typename Keys>
+__device__ __forceinline__ void group_ranks(Keys keys, int E, int K, int l, uint2* slot) {
+  float key[V];
+  int rank[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    key[v] = keys(v);
+    rank[v] = 0;
+  }
+#pragma unroll
+  for (int u = 0; u < V; ++u) {
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+      const float kj = __shfl_sync(0xffffffffu, key[u], j, G);
+#pragma unroll
+      for (int v = 0; v < V; ++v)  // false for an absent kj
+        if (u < v ? kj >= key[v] : kj > key[v] || (u == v && kj == key[v] && j < l)) ++rank[v];
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < V; ++v)
+    if (v * G + l < E && rank[v] < K) slot[rank[v]] = make_uint2(__float_as_uint(key[v]), (unsigned)(v * G + l));
+  __syncwarp();
+}
+
+// group_rounds: K rounds, each the group's best key (the lower expert of equal
+// ones) by shuffles.  For lists of four it is cheaper than counting up to K = 6
+// (T = 16384, E = 32: K = 2 2.8 us against 4.2, K = 4 3.5 against 4.2, K = 8 5.0
+// against 4.3), for lists of two up to K = 2.
+template <int V, int G, typename Keys>
+__device__ __forceinline__ void group_rounds(Keys keys, int K, int l, uint2* slot) {
+  float key[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) key[v] = keys(v);
+  for (int k = 0; k < K; ++k) {
+    float m = key[0];
+    int e = l;
+#pragma unroll
+    for (int v = 1; v < V; ++v) {
+      if (key[v] > m || m != m) {  // strictly larger: the lower expert keeps a tie
+        m = key[v];
+        e = v * G + l;
+      }
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+      const float om = __shfl_xor_sync(0xffffffffu, m, o);
+      const int oe = __shfl_xor_sync(0xffffffffu, e, o);
+      if (om > m || m != m || (om == m && oe < e)) {
+        m = om;
+        e = oe;
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      if (e == v * G + l) {
+        slot[k] = make_uint2(__float_as_uint(m), (unsigned)e);
+        key[v] = __uint_as_float(kAbsent);
+      }
+    }
+  }
+  __syncwarp();
+}
+
+template <int V, int G, typename Keys>
+__device__ __forceinline__ void token_topk(Keys keys, int E, int K, int l, uint2* slot) {
+  if constexpr (G == 32) {
+    warp_topk<V>(keys, K, l, slot);
+  } else {
+    if (V == 4 ? K <= 6 : V == 2 && K <= 2) group_rounds<V, G>(keys, K, l, slot);
+    else group_ranks<V, G>(keys, E, K, l, slot);
+  }
+}
+
+// Chosen experts per lane of a group: lane l has the k-th for k = l, l + G, ...
+template <int V, int G>
+constexpr int kPerLane = V * G <= G || G >= kMaxK ? 1 : (kMaxK + G - 1) / G;
+
+// The sum of a group's K chosen terms, w[p] of lane l being the (p G + l)-th's (0
+// from the K-th on), in that order (best expert first), in every lane: a
+// probability is a function of its chosen keys alone, not of how the lanes are
+// paired.  The shuffles of a size are in flight together; a loop to K takes them
+// one by one (8192 sequences of one token, E = 64, K = 6 90 us, now 77).
+template <int N, int P, int G>
+__device__ __forceinline__ float sum_first(const float (&w)[P]) {
   float u[N];
 #pragma unroll
-  for (int k = 0; k < N; ++k) u[k] = __shfl_sync(0xffffffffu, v, k);
+  for (int k = 0; k < N; ++k) u[k] = __shfl_sync(0xffffffffu, w[k / G], k % G, G);
   float s = 0.f;
 #pragma unroll
   for (int k = 0; k < N; ++k) s += u[k];
   return s;
 }
-__device__ __forceinline__ float sum_chosen(float v, int K) {
-  return K <= 4 ? sum_first<4>(v) : K <= 8 ? sum_first<8>(v) : sum_first<16>(v);
+template <int P, int G>
+__device__ __forceinline__ float sum_chosen(const float (&w)[P], int K) {
+  constexpr int N = P * G < kMaxK ? P * G : kMaxK;  // K is at most this
+  if (N <= 4 || K <= 4) return sum_first<(N < 4 ? N : 4), P, G>(w);
+  if (N <= 8 || K <= 8) return sum_first<(N < 8 ? N : 8), P, G>(w);
+  return sum_first<N, P, G>(w);
 }
 
 }  // namespace sel

@@ -66,7 +66,8 @@ def test_probabilities_are_summed_best_first(K):
     assert abi.moe_check_device_status() == 0
 
 
-@pytest.mark.parametrize("E,K", [(3, 3), (32, 16), (40, 8), (64, 5), (128, 16), (200, 8), (256, 16)])
+@pytest.mark.parametrize("E,K", [(3, 3), (4, 1), (7, 7), (8, 2), (9, 2), (15, 9), (16, 16), (17, 3), (24, 6),
+                                 (31, 7), (32, 16), (40, 8), (64, 5), (128, 16), (200, 8), (256, 16)])
 def test_equal_keys_in_every_place(E, K):
     """Pairs and runs of equal keys at each rank up to past the last chosen one, in
     one lane (experts 32 apart) and across lanes, and rows that hold few distinct
@@ -101,7 +102,7 @@ def test_equal_keys_in_every_place(E, K):
     assert (idx.cpu().numpy() == ref).all() and abi.moe_check_device_status() == 0
 
 
-@pytest.mark.parametrize("E", [5, 16, 20, 64, 130])
+@pytest.mark.parametrize("E", [3, 5, 16, 20, 64, 130])
 @pytest.mark.parametrize("S,GBS", [(1, 3), (4, 5), (15, 2), (17, 2), (33, 1), (63, 2), (65, 3), (100, 1)])
 def test_sigmoid_statistics_of_short_sequences(S, GBS, E):
     """Choice counts and the balance loss where a sequence does not give every warp
