@@ -226,9 +226,13 @@ static inline int k_bound(int K) { return K <= 2 ? 2 : (K <= 4 ? 4 : (K <= 8 ? 8
 // Eight warps share a token's row where fewer than 16 rows per SM are in flight
 // with one warp per token: T = 64, K = 6, D = 2048 combine 9.6 -> 4.1 us (row
 // copies alone 8.6 -> 3.6).  Above it is even (8180 rows of 4 KB) or slower (9003 rows
-// of 2 KB: fused dispatch / router backward 8 -> 16 us).
+// of 2 KB: fused dispatch / router backward 8 -> 16 us).  Rows of much less than one
+// step of eight warps (256 vectors) leave warps idle, which K = 1 feels from 12
+// tokens per SM on: rows of 2 KB, one warp -> eight, combine backward 1600 tokens
+// 10.6 -> 10.3 us, 2000 9.8 -> 10.7, 2400 9.9 -> 11.9; rows of 4 KB 13.9 -> 13.6 at
+// 2400.
 static inline int row_parts(const Ctx& c, int64_t T, int K, int vpr) {
-  return vpr >= 128 && T * K < (int64_t)c.num_sms * 16 ? 8 : 1;
+  return vpr >= 128 && T * K < (int64_t)c.num_sms * 16 && (vpr >= 192 || T < (int64_t)c.num_sms * 12) ? 8 : 1;
 }
 // Token and part of this warp: the parts of a token are consecutive warps of one
 // block of 8, which then holds that token alone.

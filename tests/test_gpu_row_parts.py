@@ -1,5 +1,5 @@
 """The row movers with a token's row split over several warps (few tokens, rows of
-64 vectors and more) and the dispatch that ranks and copies in one launch (up to
+128 vectors and more) and the dispatch that ranks and copies in one launch (up to
 512 slots), against float64: combine and its backward, the dispatch
 backward, and the fused dispatch / router backward.  bf16 results are one
 rounding of an fp32 sum (2^-9); fp32 sums of n terms stay within n 2^-24 of
@@ -19,7 +19,8 @@ def _rel(a, b):
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("T,K,E,D", [(1, 1, 4, 64), (3, 2, 5, 512), (13, 4, 33, 1088), (9, 8, 64, 2560),
                                      (7, 16, 100, 2048), (73, 7, 64, 576), (128, 4, 31, 1024),
-                                     (171, 3, 256, 512), (512, 1, 2, 64), (1830, 3, 40, 1024), (3700, 2, 8, 512)])
+                                     (171, 3, 256, 512), (512, 1, 2, 64), (1830, 3, 40, 1024), (3700, 2, 8, 512),
+                                     (1823, 1, 16, 512), (1825, 1, 16, 1024), (2431, 1, 4, 2048)])
 def test_row_movers(T, K, E, D, dtype):
     import __graft_entry__
     __graft_entry__.build()
