@@ -151,12 +151,13 @@ cudaError_t launch_dispatch_fp8(const Ctx& c, const void* x, const int32_t* row_
 cudaError_t launch_dequant_rows(const Ctx& c, const void* xq, const float* scale, int64_t rows, int D, void* out) {
   if (rows == 0) return cudaSuccess;
   const int vpr = D / 8;
-  const int L = vpr >= 32 ? 32 : vpr >= 16 ? 16 : 8;
+  const int L = dequant_lanes(c, rows, vpr);
   const int rpb = 256 / L;
   const unsigned blocks = (unsigned)((rows + rpb - 1) / rpb);
   const uint2* q = (const uint2*)xq;
   KernelScope ks("dequant_rows", c.stream);
-  if (L == 32) dequant_rows_kernel<32><<<blocks, 256, 0, c.stream>>>(q, scale, rows, vpr, (uint4*)out);
+  if (L == 256) dequant_rows_kernel<256><<<blocks, 256, 0, c.stream>>>(q, scale, rows, vpr, (uint4*)out);
+  else if (L == 32) dequant_rows_kernel<32><<<blocks, 256, 0, c.stream>>>(q, scale, rows, vpr, (uint4*)out);
   else if (L == 16) dequant_rows_kernel<16><<<blocks, 256, 0, c.stream>>>(q, scale, rows, vpr, (uint4*)out);
   else dequant_rows_kernel<8><<<blocks, 256, 0, c.stream>>>(q, scale, rows, vpr, (uint4*)out);
   return cudaGetLastError();

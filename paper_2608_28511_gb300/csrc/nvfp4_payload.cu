@@ -171,9 +171,9 @@ __global__ void __launch_bounds__(256) dispatch_nvfp4_kernel(const uint4* __rest
 }
 
 // x_perm[r] = code * s_b * g in bf16 (exact), 8 elements (4 code bytes, one
-// 16-byte store) per thread step.  L lanes per row (32, fewer for rows shorter
-// than 32 vectors), four steps' loads in flight before the first is converted,
-// so no address needs a division and a warp writes 512 contiguous bytes.
+// 16-byte store) per thread step.  L lanes per row (dequant_lanes), four steps'
+// loads in flight before the first is converted, so no address needs a division
+// and a warp writes 512 contiguous bytes.
 // Bound by HBM: at 49146 rows of 2048 (258 MB) 37.4 us, 6.9 TB/s; one step per
 // thread of a flat grid, with a 64-bit division for the row, took 60.
 template <int L>
@@ -244,12 +244,13 @@ cudaError_t launch_dequant_nvfp4(const Ctx& c, const void* xq, const uint8_t* bs
                                  int64_t rows, int D, void* out) {
   if (rows == 0) return cudaSuccess;
   const int vpr = D / 8;  // a multiple of 8
-  const int L = vpr >= 32 ? 32 : vpr >= 16 ? 16 : 8;
+  const int L = dequant_lanes(c, rows, vpr);
   const int rpb = 256 / L;
   const unsigned blocks = (unsigned)((rows + rpb - 1) / rpb);
   const uint32_t* q = (const uint32_t*)xq;
   KernelScope ks("dequant_nvfp4", c.stream);
-  if (L == 32) dequant_nvfp4_kernel<32><<<blocks, 256, 0, c.stream>>>(q, bscale, rscale, rows, vpr, (uint4*)out);
+  if (L == 256) dequant_nvfp4_kernel<256><<<blocks, 256, 0, c.stream>>>(q, bscale, rscale, rows, vpr, (uint4*)out);
+  else if (L == 32) dequant_nvfp4_kernel<32><<<blocks, 256, 0, c.stream>>>(q, bscale, rscale, rows, vpr, (uint4*)out);
   else if (L == 16) dequant_nvfp4_kernel<16><<<blocks, 256, 0, c.stream>>>(q, bscale, rscale, rows, vpr, (uint4*)out);
   else dequant_nvfp4_kernel<8><<<blocks, 256, 0, c.stream>>>(q, bscale, rscale, rows, vpr, (uint4*)out);
   return cudaGetLastError();

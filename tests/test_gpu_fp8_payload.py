@@ -135,3 +135,17 @@ def test_fp8_payload_rejects_fp32():
                              z(16, d=torch.int32), z(16, d=torch.int32), z(16, 64, d=torch.uint8), z(16), z(16),
                              z(1 << 16, d=torch.uint8))
     assert e.value.status == -8
+
+
+@pytest.mark.parametrize("R,D", [(1, 64), (1, 1088), (7, 1024), (20, 4160), (607, 2112), (608, 2112)])
+def test_receiver_of_few_rows(R, D):
+    """moe_dequant_rows with a warp or a block per row, on both sides of four rows
+    per SM, with rows that end inside a round: every finite code times the scale."""
+    from paper_2608_28511_gb300 import abi
+    g = torch.Generator().manual_seed(R + D)
+    codes = torch.randint(0, 127, (R, D), generator=g) + 128 * torch.randint(0, 2, (R, D), generator=g)
+    codes, scale = codes.to(torch.uint8), torch.pow(2.0, torch.randint(-20, 20, (R,), generator=g).float())
+    out = torch.full((R + 1, D), 7.0, dtype=torch.bfloat16, device="cuda")
+    abi.moe_dequant_rows(abi.MoeShape.of(R, 1, 1, D, 4, 64), codes.cuda(), scale.cuda(), out[:R])
+    assert np.array_equal(f64(out[:R]), O.fp8_dequantize_rows(codes.numpy(), scale.double().numpy()))
+    assert bool((out[R] == 7.0).all())

@@ -237,3 +237,11 @@ def test_infinities_saturate_with_their_sign(D):
     got = np.empty_like(want)
     got[:, 0::2], got[:, 1::2] = q & 0xF, q >> 4
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("T,D", [(1, 64), (1, 1024), (1, 1088), (3, 2048), (5, 4160), (151, 2112), (152, 2112), (153, 1088)])
+def test_receiver_of_few_rows(T, D):
+    """A warp or a block per received row on both sides of four rows per SM (K = 4),
+    with rows that end inside a round."""
+    g = torch.Generator().manual_seed(T * D)
+    _check_direct(torch.randn(T, D, generator=g).to(torch.bfloat16), K=4, E=8)
