@@ -11,6 +11,8 @@
 #include <cuda_fp8.h>
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "launch.h"
 
@@ -93,7 +95,10 @@ __device__ __forceinline__ void quantize_block(const uint4& v0, const uint4& v1,
 // One warp per token: the row maximum and scale, then every block's scale and
 // codes, written to each of the token's K rows (row_of_slot).  NB > 0: a lane's
 // (at most NB) blocks are read once, into registers; wider rows are read twice.
-// T = 8191, K = 6, D = 2048, dispatch and arrival: 69.8 -> 67.8 us.
+// T = 8191, K = 6, D = 2048, dispatch and arrival: 69.8 -> 67.8 us.  NB is no larger
+// than the row needs, since the unused blocks cost their share of the code (with
+// the permutation, warm, T = 8191, K = 6: D = 256 read twice 15.9 us, NB = 4 18.1,
+// NB = 1 14.2; D = 1024 18.5, 20.7, NB = 2 18.0).
 template <int KM, int NB>
 __global__ void __launch_bounds__(256) dispatch_nvfp4_kernel(const uint4* __restrict__ x,
                                                              const int32_t* __restrict__ row_of_slot, int64_t T,
@@ -230,12 +235,18 @@ cudaError_t launch_dispatch_nvfp4(const Ctx& c, const void* x, const int32_t* ro
     kernel<<<grid, 32 * warps, 0, c.stream>>>((const uint4*)x, row_of_slot, T, K, vpr, (uint2*)xq, bscale, rscale,
                                               c.err);
   };
-  const bool regs = D <= 2048;
+  auto by_width = [&](auto km) {
+    constexpr int KM = decltype(km)::value;
+    if (D <= 512) run(dispatch_nvfp4_kernel<KM, 1>);
+    else if (D <= 1024) run(dispatch_nvfp4_kernel<KM, 2>);
+    else if (D <= 2048) run(dispatch_nvfp4_kernel<KM, 4>);
+    else run(dispatch_nvfp4_kernel<KM, 0>);
+  };
   switch (k_bound(K)) {
-    case 2: regs ? run(dispatch_nvfp4_kernel<2, 4>) : run(dispatch_nvfp4_kernel<2, 0>); break;
-    case 4: regs ? run(dispatch_nvfp4_kernel<4, 4>) : run(dispatch_nvfp4_kernel<4, 0>); break;
-    case 8: regs ? run(dispatch_nvfp4_kernel<8, 4>) : run(dispatch_nvfp4_kernel<8, 0>); break;
-    default: regs ? run(dispatch_nvfp4_kernel<16, 4>) : run(dispatch_nvfp4_kernel<16, 0>); break;
+    case 2: by_width(std::integral_constant<int, 2>()); break;
+    case 4: by_width(std::integral_constant<int, 4>()); break;
+    case 8: by_width(std::integral_constant<int, 8>()); break;
+    default: by_width(std::integral_constant<int, 16>()); break;
   }
   return cudaGetLastError();
 }

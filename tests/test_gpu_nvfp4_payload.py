@@ -194,7 +194,7 @@ def test_midpoints_of_every_block_scale(exp):
     _check_direct(torch.stack([x, -x]).to(torch.bfloat16), K=1, E=4)
 
 
-@pytest.mark.parametrize("D", [64, 576, 1984, 2048, 2112, 2560])
+@pytest.mark.parametrize("D", [64, 512, 576, 1024, 1088, 1984, 2048, 2112, 2560])
 def test_row_widths_around_the_register_path(D):
     """Rows that a lane's registers hold and wider ones, whole and partial last
     rounds of 32 blocks."""
