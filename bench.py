@@ -49,6 +49,10 @@ def _peaks() -> dict:
 # once and each result written once.
 # ---------------------------------------------------------------------------
 
+# The kernels whose time the row movement's rate is quoted on.
+PERM_KERNELS = ("dispatch_rows", "perm_dispatch", "combine", "combine_bwd", "dispatch_bwd", "dispatch_route_bwd")
+
+
 def kernel_work(name: str, w: synth.Workload, T: int, Fs: int = 0, latent_fused: bool = False) -> tuple[str, float]:
     """(bound, algorithmic work per launch) of a library kernel: flops for the
     tensor-core GEMMs, bytes for the rest.  latent_fused: the LatentMoE dgrad
@@ -59,6 +63,7 @@ def kernel_work(name: str, w: synth.Workload, T: int, Fs: int = 0, latent_fused:
     flops = {
         "ffn1_swiglu": 4.0 * TK * D * F, "ffn2": 2.0 * TK * F * D, "ffn2_dgrad": 2.0 * TK * D * F,
         "ffn2_dgrad_swiglu": 2.0 * TK * D * F, "ffn2_wgrad": 2.0 * TK * D * F, "ffn1_dgrad": 4.0 * TK * F * D, "ffn1_wgrad": 4.0 * TK * F * D,
+        "ffn_bwd": 10.0 * TK * D * F,  # fp32: both weight gradients and GEMM-1's dgrad in one launch
         "latent_fwd": 2.0 * T * w.H * D, "latent_dgrad": 2.0 * T * w.H * (D + (E if latent_fused else 0)),
         "latent_wgrad": 2.0 * T * w.H * D,
         "router_dgrad": 2.0 * T * Din * E, "router_wgrad": 2.0 * T * Din * E,
@@ -88,9 +93,9 @@ def kernel_work(name: str, w: synth.Workload, T: int, Fs: int = 0, latent_fused:
         "dequant_rows": TK * D + TK * D * bx + 4 * TK,
         "dispatch_nvfp4": T * D * bx + TK * (D // 2 + D // 16) + 8 * TK,
         "dequant_nvfp4": TK * (D // 2 + D // 16) + TK * D * bx + 4 * TK,
-        "pack_w1": 0.0,
+        "pack_w1": 0.0, "perm_zero": 0.0, "group_maps": 0.0, "sum_splits": 0.0,  # (the splits are not the method's)
     }
-    return "hbm", float(byts.get(base, 0.0))
+    return "hbm", float(byts[base])
 
 
 def gemm_bytes(name: str, w: synth.Workload, T: int, Fs: int = 0, latent_fused: bool = False) -> float:
@@ -111,6 +116,7 @@ def gemm_bytes(name: str, w: synth.Workload, T: int, Fs: int = 0, latent_fused: 
         "ffn2_wgrad": (TK * F + TK * D) * bx + E * D * F * 4,
         "ffn1_dgrad": (TK * 2 * F + E * 2 * F * D + TK * D) * bx,
         "ffn1_wgrad": (TK * 2 * F + TK * D) * bx + E * 2 * F * D * 4,
+        "ffn_bwd": (TK * 3 * F + 3 * TK * D + E * 2 * F * D) * bx + 3 * E * D * F * 4,
         # the two projections (down: x -> x_lat, up: y_lat -> y) move the same bytes
         "latent_fwd": (T * H + H * D + T * D) * bx,
         "latent_dgrad": (T * (D + (E if latent_fused else 0)) + (D + (E if latent_fused else 0)) * H + T * H) * bx,
@@ -625,8 +631,7 @@ def main() -> None:
     roof = top_roofline(kernels, w, peaks)
 
     exp_ms = sum(v["ms_per_step"] for k, v in kernels.items() if k.startswith("ffn"))
-    perm_names = ("dispatch_rows", "combine", "combine_bwd", "dispatch_bwd", "dispatch_route_bwd")
-    perm_ms = sum(v["ms_per_step"] for k, v in kernels.items() if k in perm_names)
+    perm_ms = sum(v["ms_per_step"] for k, v in kernels.items() if k in PERM_KERNELS)
 
     # ---- the other workloads, device-timed only (1 GPU)
     per_workload = None
