@@ -197,10 +197,10 @@ int router_splits(const Dims& d, int num_sms) {
 }
 // The same for the CUDA-core engine (fp32 inputs, or a number of experts that
 // the tensor-core engine does not take).  Up to 32 experts: 32 x 32 tiles, the
-// three blocks per SM that fit, each reducing at least 256 tokens.  More: enough
-// splits for two 64 x 128 tiles per SM, which do twice the products per staged
-// element, down to 128 tokens: bf16 T = 2045, E = 60, Din = 2048 41 us on 32 x 32
-// tiles, 23 now.
+// three blocks per SM that fit, each reducing at least 256 tokens.  More: splits for
+// two 64 x 128 tiles per SM, which do twice the products per staged element, down
+// to 128 tokens: bf16 T = 2045, E = 60, Din = 2048 41 us on 32 x 32 tiles, 23 now
+// (where kRouterSplits is too few for that, the engine takes a smaller tile).
 int router_splits_simt(const Dims& d, int num_sms) {
   const bool thin = d.E <= 32;
   const int64_t tiles = thin ? (d.Din + 31) / 32 : (int64_t)((d.E + 63) / 64) * ((d.Din + 127) / 128);

@@ -444,6 +444,10 @@ cudaError_t run(const Ctx& c, const GemmDesc (&ds)[NP]) {
   const bool swiglu = ds[0].epi == Epi::SwigluFwd;  // needs gate and up columns in one 128-column tile
   int64_t widest = 0;
   for (const GemmDesc& d : ds) widest = d.N > widest ? d.N : widest;
+  // a split reduction onto at most 32 rows (router_splits_simt sizes the splits for
+  // this tile): a taller tile is half empty.  fp32, E = 12, Din = 1024, T = 4096 35.0
+  // us on 64 x 64 tiles, 31.5 here; Din = 2048 53 and 45
+  if (NP == 1 && ds[0].group == Group::K && ds[0].M <= 32) return run_tile<TA, TB, TC, 32, 32, 32>(c, ds);
   if constexpr (sizeof(TA) == 4 && sizeof(TB) == 4) {
     // the largest tile that still gives every SM work: at T = 256, D = 128, E = 8,
     // K = 2, F = 256 the small tiles take GEMM-1's dgrad from 102 to 17 us

@@ -49,7 +49,7 @@ def test_fp32_projection(T, n_in, n_out, accumulate):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("T,E,D", [(1, 3, 64), (511, 5, 128), (513, 13, 192), (3001, 60, 256), (5000, 129, 64),
-                                   (4096, 12, 512)])
+                                   (4096, 12, 512), (4096, 12, 1024), (3700, 31, 2048), (2100, 33, 1088)])
 def test_router_with_odd_experts(T, E, D, dtype):
     """Logits, and the weight gradient with and without the split over tokens."""
     K = min(3, E)
