@@ -1,7 +1,8 @@
-"""The fp32 expert backward, whose three products that depend on dH run in one
+"""The fp32 expert block: the forward on each of the tiles that its SwiGLU epilogue
+takes (32, 64 and 128 rows of 128 columns), and the backward, whose three products that depend on dH run in one
 launch and whose SwiGLU backward runs in the epilogue of dA's product, on every
 tile size that the row counts select, with empty experts.  Each output against
-float64 from the GPU's own h and a; a sum of n fp32 products is within
+float64, those after h and a from the GPU's own; a sum of n fp32 products is within
 n 2^-24 of sum |a b|, about sqrt(n) 2^-24 of the result's norm for random signs,
 and dH carries the sum over D and about ten roundings of its own: four times the
 sum of both is allowed."""
@@ -19,7 +20,7 @@ EDGES = [0, 1, 31, 32, 33, 0, 63, 64, 65, 130]
 
 @pytest.mark.parametrize("counts,D,F", [([1], 64, 64), (EDGES, 64, 64), (EDGES, 192, 128), (EDGES, 64, 1216),
                                         ([0, 700, 129, 1], 512, 448), ([5] * 40, 128, 192),
-                                        ([900, 0, 1, 1100], 320, 768)])
+                                        ([900, 0, 1, 1100], 320, 768), ([300, 0, 150, 50], 128, 1216)])
 def test_fp32_expert_backward(counts, D, F):
     import __graft_entry__
     __graft_entry__.build()
@@ -48,6 +49,9 @@ def test_fp32_expert_backward(counts, D, F):
         he = h[r].double().view(n, F // 64, 2, 64)
         gate, up = he[:, :, 0].reshape(n, F), he[:, :, 1].reshape(n, F)
         s = torch.sigmoid(gate)
+        near(h[r], x[r].double() @ w1[e].double().T, D)
+        near(act[r], gate * s * up, 1)
+        near(y[r], act[r].double() @ w2[e].double().T, F)
         dA = dy[r].double() @ w2[e].double()
         dg, du = dA * up * s * (1 + gate * (1 - s)), dA * gate * s
         dH = torch.stack([dg.view(n, F // 64, 64), du.view(n, F // 64, 64)], 2).reshape(n, 2 * F)

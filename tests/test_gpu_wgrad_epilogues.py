@@ -3,7 +3,8 @@ select (stores by the copy engine, by eight and by four epilogue warps), with
 empty and ragged experts and widths that end inside a tile.  dw2 against float64
 products of the same bf16 operands: a sum of n products in fp32 is within
 n 2^-24 of sum |a b|, about sqrt(n) 2^-24 of the norm, of which four times is
-allowed; dw1's operand dH is rounded to bf16 from a hardware tanh (2^-7)."""
+allowed; dw1's operand dH, which dx_perm shares, is rounded to bf16 from a
+hardware tanh (2^-7)."""
 import itertools
 
 import pytest
@@ -50,5 +51,5 @@ def test_weight_gradients(form, D, F):
         dA = dy[r].double() @ w2[e].double()
         dg, du = dA * up * s * (1 + gate * (1 - s)), dA * gate * s
         dH = torch.stack([dg.view(n, F // 64, 64), du.view(n, F // 64, 64)], 2).reshape(n, 2 * F)
-        ref = dH.T @ x[r].double()
-        assert float((dw1[e].double() - ref).norm() / ref.norm()) < 2.0 ** -7, (e, n)
+        for got, ref in ((dw1[e], dH.T @ x[r].double()), (dx[r], dH @ w1[e].double())):
+            assert float((got.double() - ref).norm() / ref.norm()) < 2.0 ** -7, (e, n)
