@@ -96,10 +96,10 @@ int moe_workspace_size(const moe_shape_t* shape, size_t* bytes);
 int moe_route(const moe_shape_t* shape, const void* x, const void* w_router, const float* bias,
               float* logits, int32_t* topk_idx, float* topk_prob, void* ws, size_t ws_bytes, void* stream);
 
-/* Top-K of given fp32 logits [T, E]: the K largest
- * logits (ties to the lower expert index), ordered by descending logit, and
- * renormalised probabilities p_k = exp(z_k - z_max) / sum over the K chosen
- * (equal to softmax over all E restricted to the chosen set). */
+/* Top-K of given fp32 logits [T, E]: the K largest logits (ties to the lower
+ * expert index), ordered by descending logit, and renormalised probabilities
+ * p_k = exp(z_k - z_max) / sum over the K chosen, added in that order (equal to
+ * softmax over all E restricted to the chosen set). */
 int moe_topk(const moe_shape_t* shape, const float* logits, int32_t* topk_idx, float* topk_prob, void* stream);
 
 /* Dispatch (forward hidden and probability transfers, Sec. 4.1 footnote):
@@ -225,7 +225,8 @@ int moe_combine_bwd(const moe_shape_t* shape, const void* dy, const void* y_perm
  * dx_perm = dH . w1_e, dw2_e = dy_perm_e^T . a_e, dw1_e = dH_e^T . x_perm_e.
  * dw1 [E, 2F, D] and dw2 [E, D, F] are fp32 and fully written (zero for an
  * expert with no rows).  dH [TK, 2F] lives in the workspace.  The SwiGLU
- * backward runs in dA's GEMM on its fp32 accumulator (dA is never stored). */
+ * backward runs in dA's GEMM on its fp32 accumulator (dA is never stored).
+ * dx_perm may take the place of dy_perm, x_perm or act_save. */
 int moe_expert_ffn_bwd(const moe_shape_t* shape, const void* dy_perm, const void* x_perm, const void* h_save,
                        const void* act_save, const int32_t* expert_offsets, const void* w1, const void* w2,
                        void* dx_perm, float* dw1, float* dw2, void* ws, size_t ws_bytes, void* stream);

@@ -17,7 +17,7 @@
 namespace moe {
 
 // Scratch of the counting sort: E * ceil(T*K / 2048) int32 per-chunk counts
-// (counts[e * nchunks + chunk]).
+// (counts[chunk * E + e]).
 static __device__ __align__(256) int32_t g_dispatch_scratch[MOE_DISPATCH_NOALLOC_SCRATCH_INTS];
 
 namespace {
@@ -74,8 +74,9 @@ extern "C" int moe_dispatch_noalloc(const moe_shape_t* shape, const void* x, con
   int32_t* scratch = nullptr;
   st = scratch_for_device(c.device, &scratch);
   if (st != MOE_OK) return st;
-  // Every table entry the kernels read is written earlier in the same call
-  // (the histogram writes all E x chunks counts), so no clearing is needed.
+  // Every table entry the kernels read is written earlier in the same call (the
+  // histogram writes all E x chunks counts; a single chunk needs no table), so no
+  // clearing is needed.
   if (x_perm)
     return abi_cuda_status(launch_permute_dispatch(c, x, topk_idx, topk_prob, d.T, d.K, d.E, (int64_t)d.D * d.bx,
                                                    expert_offsets, row_of_slot, token_of_row, prob_perm, x_perm,

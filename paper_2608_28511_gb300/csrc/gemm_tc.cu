@@ -150,9 +150,12 @@ bool make_plan(const GemmDesc& d, Plan* pl) {
 // an equal share: the tiles of n full-height rounds over the pairs are cut down
 // to one height, in whole 8-row swizzle atoms.  With 128-row tiles on single
 // CTAs a batch of 8192 ran on 64 SMs and one of 30011 took two uneven rounds,
-// and every tile copied all of W_r; a pair's CTAs copy half each.  T = 30011,
-// E = 128, D = 2048 (139 MB): 27.0 -> 24.1 us; T = 2045, E = 60: 10.7 -> 9.7;
-// T = 16384, E = 256, 4096 wide: 36 -> 31; T = 8192, E = 64: 10.9 -> 11.7.
+// and every tile copied all of W_r; a pair's CTAs copy half each.  Cold L2, with
+// the elected MMA issue below, single CTAs -> pairs: T = 30011, E = 128, D = 2048
+// (139 MB) 37.8 -> 35.1 us; T = 2045, E = 60 18.5 -> 13.7; T = 16384, E = 256, 4096
+// wide 49.0 -> 42.5; T = 8192, E = 64 18.8 -> 16.7.  Even at T = 16384, E = 64 (22.8,
+// 22.9); up to 1 us longer where there is little to copy (E = 8, D = 256, T = 9728
+// 9.5 -> 10.5).
 int router_tile_rows(int64_t M, int num_sms) {
   const int64_t slots = num_sms / 2 * 2;
   const int64_t rounds = (M + slots * BM - 1) / (slots * BM);
@@ -369,9 +372,19 @@ cudaError_t launch_gemm_tc(const Ctx& c, const GemmDesc& d, const char* name, co
       // D = 2048, F = 1408, E = 60 (0.69 and 1.38 GB), stored by eight warps -> by the
       // copy engine: 17 rows per expert 133 -> 121 and 234 -> 215 us, 136 rows 138 ->
       // 126 and 244 -> 232, 256 rows 146 -> 136 and 255 -> 248, 384 rows 156 -> 156
-      // and 276 -> 295 (the loads miss the stage).
+      // and 276 -> 295 (the loads miss the stage).  Other widths at 160 to 240 rows:
+      // D = 2048, F = 1024, E = 128 200 -> 191 and 379 -> 361, D = 1024, F = 768, E = 256
+      // 158 -> 151 and 292 -> 286, D = 1408, F = 704, E = 60 62 -> 54 and 113 -> 96,
+      // D = 2560, F = 1536, E = 8 38 -> 33 and 62 -> 54.  Against the form before both
+      // (four warps, MMAs not issued by one elected lane), counts that average under
+      // the line with one expert of most rows gain as well (three quarters of 256 rows
+      // on average, E = 256: whole expert backward 1402 -> 1278 us), and counts that are
+      // all multiples of 64 lose: nothing holds the CTA pairs together then, they drift
+      // apart under the stores, and the operands are read twice from memory (E = 256,
+      // 192 rows: 457 MB instead of 251; GEMM-1's 320 -> 357 us, of 128 experts 422 ->
+      // 447, of 60 277 -> 282; at 320 rows and eight warps 330 -> 388).
       if (d.offsets && d.max_rows <= 4 * (int64_t)tc::BK * d.num_groups && d.M % 64 == 0 && d.N % 64 == 0 &&
-          d.sc_g % 4 == 0 && make_store_map(&p.tc, d))
+          d.ldc == d.N && d.sc_g == d.M * d.N && make_store_map(&p.tc, d))
         return launch_inst<256, true, true, 2, 0, float, 2, 0, tc::kBulkEpi>(c, p, ub);
       // Short groups (up to ten): eight epilogue warps.  Four warps -> eight: 512
       // rows (D = 1024, F = 768, E = 256) 204 -> 201 and 373 -> 373 us, 546 rows

@@ -423,7 +423,7 @@ struct Cfg {
   static constexpr int kABytes = BM * BK * 2;
   static constexpr int kBBytes = kBRows * BK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  // Bulk-store epilogue (weight gradients of short groups, EWF = 8)
+  // Bulk-store epilogue (weight gradients of short groups)
   static constexpr bool kBulk = TCB == 4 && EWF == kBulkEpi;
   // EPI 5 (SwiGLU backward) gives one stage to its h slots, the bulk-store
   // epilogue one to its staging
@@ -1273,13 +1273,7 @@ __global__ void __launch_bounds__(
       uint8_t* c_rows = reinterpret_cast<uint8_t*>(Cb) + rbase * ldc_b;
       if (ti.nkb == 0) {
         // an expert with no rows: its weight-gradient tile is zero
-        if (C::kBulk) {
-          for (int c = ch; c < BN / 32; c += CSTEP) {
-            const int64_t col = n0 + c * 32 + lane;
-            for (int r = 0; r < nrows && col < N; ++r) Cb[(rbase + r) * ldc + col] = from_f32<TC>(0.f);
-          }
-          continue;
-        }
+        if (C::kBulk) continue;  // written by the zero warp (the form is chosen for contiguous groups only)
         uint4 z[NP];
 #pragma unroll
         for (int i = 0; i < NP; ++i) z[i] = make_uint4(0, 0, 0, 0);

@@ -186,8 +186,8 @@ struct GemmDesc {
 };
 
 cudaError_t launch_gemm_simt(const Ctx& c, const GemmDesc& d, const char* name);
-// Three independent fp32 products in one launch; the longest reduction comes
-// first, so that the short ones fill in behind it.
+// Three independent fp32 products in one launch, each product's blocks behind the
+// one before's.
 cudaError_t launch_gemm_simt_f32x3(const Ctx& c, const GemmDesc (&ds)[3], const char* name);
 
 // tcgen05 / TMA engine (bf16 operands only).  Returns cudaErrorNotSupported

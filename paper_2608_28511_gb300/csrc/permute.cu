@@ -560,6 +560,8 @@ __global__ void __launch_bounds__(256, KM <= 8 ? 3 : 1) dispatch_route_bwd_kerne
     }
     st_stream(dx + t * vpr + v, pack16<T>(acc));
   }
+  // (held over the loop below it costs P = 1 a third of its speed)
+  if (P == 1 && lane < K) dprob[t * K + lane] = my_dp;
   for (int e0 = part * 32; e0 < E; e0 += 32 * P) {
     const int e = e0 + lane;
     float val = 0.f;
@@ -571,9 +573,10 @@ __global__ void __launch_bounds__(256, KM <= 8 ? 3 : 1) dispatch_route_bwd_kerne
       if (dz16) dz16[t * E + e] = __float2bfloat16_rn(val);
     }
   }
-  // dprob may lie over prob, which all parts have used by then
-  if (P > 1) __syncthreads();
-  if (part == 0 && lane < K) dprob[t * K + lane] = my_dp;
+  if (P > 1) {  // dprob may lie over prob, which all parts have used by then
+    __syncthreads();
+    if (part == 0 && lane < K) dprob[t * K + lane] = my_dp;
+  }
 }
 
 cudaError_t launch_dispatch_route_bwd(const Ctx& c, DType dt, const void* dx_perm, const float* dprob_perm,
