@@ -38,9 +38,10 @@ constexpr int kSelWarps = 16;
 // 10.4 us, 13.6 with eight warps; staging 64 rows in shared memory and selecting
 // with four threads per token took 14.3.  E = 8, K = 2, T = 16384 with the balance
 // statistics: 11.2 us with a warp per token, 8.3 with groups.
-// At least two blocks per SM (64 registers a thread; V = 8 takes 74 by itself:
-// T = 16384, E = 256, K = 8 33 -> 27 us), three for short lists (40 registers, not
-// 50).
+// At least two blocks per SM, three for short lists (40 registers, not 50).  V = 8
+// has 64 registers for it with its biases in shared memory: T = 16384, E = 256, K = 8
+// 29 us with one block, 27 with the biases in registers (which spill, and cost a
+// single sequence of 64 tokens 10.0 -> 11.1), 23 now (9.7).
 template <int V, int G>
 __global__ void __launch_bounds__(32 * kSelWarps, V <= 2 ? 3 : 2) select_sigmoid_kernel(
     const float* __restrict__ logits, const float* __restrict__ bias, int64_t S, int E, int K, int tpb, int nch,
@@ -51,19 +52,24 @@ __global__ void __launch_bounds__(32 * kSelWarps, V <= 2 ? 3 : 2) select_sigmoid
   __shared__ float wsum[kSelWarps][V * 32];
   __shared__ uint2 slots[kSelWarps][TW][kMaxK];
   __shared__ int cnt[V * 32];
+  constexpr bool kSharedBias = V == 8;
+  __shared__ float s_b[kSharedBias ? V * G : 1];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ch = blockIdx.x, g = blockIdx.y;
   const int sub = lane / G, l = lane % G;
   const int64_t t0 = (int64_t)g * S + (int64_t)ch * tpb;
   const int n = (int)min((int64_t)tpb, S - (int64_t)ch * tpb);
   for (int e = tid; e < V * 32; e += 32 * kSelWarps) cnt[e] = 0;
+  if (kSharedBias)
+    for (int e = tid; e < V * G; e += 32 * kSelWarps) s_b[e] = bias && e < E ? __ldg(bias + e) : 0.f;
   if (ch == 0 && g == 0 && tid == 0) *ticket = 0u;  // for the finalize kernel that follows
   __syncthreads();
-  float b[V], acc[V], z[V];
+  float b[kSharedBias ? 1 : V], acc[V], z[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    b[v] = bias && v * G + l < E ? __ldg(bias + v * G + l) : 0.f;
+    if (!kSharedBias) b[v] = bias && v * G + l < E ? __ldg(bias + v * G + l) : 0.f;
     acc[v] = 0.f;
   }
+  auto bias_of = [&](int v) { return kSharedBias ? s_b[v * G + l] : b[kSharedBias ? 0 : v]; };
   auto fetch = [&](int q) {
 #pragma unroll
     for (int v = 0; v < V; ++v)
@@ -80,7 +86,7 @@ __global__ void __launch_bounds__(32 * kSelWarps, V <= 2 ? 3 : 2) select_sigmoid
     for (int v = 0; v < V; ++v) {
       const bool in = v * G + l < E;
       s[v] = in ? sigmoidf_(z[v]) : 0.f;
-      if (keys && in && live) keys[t * E + v * G + l] = __fadd_rn(s[v], b[v]);
+      if (keys && in && live) keys[t * E + v * G + l] = __fadd_rn(s[v], bias_of(v));
       ssum += s[v];
     }
     if (q + TW < q1) fetch(q + TW + sub);
@@ -89,7 +95,7 @@ __global__ void __launch_bounds__(32 * kSelWarps, V <= 2 ? 3 : 2) select_sigmoid
     const uint2* slot = slots[warp][sub];
     sel::token_topk<V, G>(
         [&](int v) {
-          return v * G + l < E ? sel::key_of(__fadd_rn(s[v], b[v])) : __uint_as_float(sel::kAbsent);
+          return v * G + l < E ? sel::key_of(__fadd_rn(s[v], bias_of(v))) : __uint_as_float(sel::kAbsent);
         },
         E, K, l, slots[warp][sub]);
     // the chosen experts' scores, from the lanes that hold them
