@@ -46,11 +46,16 @@ __global__ void __launch_bounds__(256) topk_kernel(const float* __restrict__ log
 cudaError_t launch_topk(const Ctx& c, const float* logits, int64_t T, int E, int K, int32_t* idx, float* prob) {
   if (T == 0) return cudaSuccess;
   KernelScope ks("topk", c.stream);
-  sel::for_experts(E, [&](auto v, auto g) {
+  auto run = [&](auto v, auto g) {
     constexpr int G = decltype(g)::value, per = 8 * 32 / G;  // tokens per block
     topk_kernel<decltype(v)::value, G>
         <<<(unsigned)((T + per - 1) / per), 256, 0, c.stream>>>(logits, T, E, K, idx, prob);
-  });
+  };
+  // 17 to 32 experts: while the GPU holds all warps at once, the shorter chain of a
+  // warp per token is faster (E = 32, warm, groups of eight lanes -> warps: T = 1024,
+  // K = 4 2.2 -> 1.8 us, K = 8 2.7 -> 1.9; T = 16384, K = 4 3.5 -> 4.0)
+  if (E > 16 && E <= 32 && T <= 4096) run(std::integral_constant<int, 1>(), std::integral_constant<int, 32>());
+  else sel::for_experts(E, run);
   return cudaGetLastError();
 }
 

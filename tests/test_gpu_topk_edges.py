@@ -128,3 +128,17 @@ def test_sigmoid_statistics_of_short_sequences(S, GBS, E):
     P = (s / s.sum(1, keepdim=True)).view(GBS, S, E).mean(1)
     want = 0.5 / GBS * float((cnt * E / (K * S) * P).sum())
     assert abs(float(loss[0]) - want) <= 2e-6 * abs(want)
+
+
+@pytest.mark.parametrize("T", [4096, 4097])
+@pytest.mark.parametrize("E,K", [(17, 3), (32, 8)])
+def test_both_forms_for_up_to_32_experts(T, E, K):
+    """A warp per token up to 4096 tokens, eight lanes per token above: the same
+    indices and bits of the probabilities for the rows that both have."""
+    z = torch.round(torch.randn(8000, E, generator=torch.Generator().manual_seed(T)) * 8) / 8
+    idx, prob = torch.empty(8000, K, dtype=torch.int32, device="cuda"), torch.empty(8000, K, device="cuda")
+    abi.moe_topk(abi.MoeShape.of(8000, 1, K, 64, E, 64), z.cuda(), idx, prob)
+    i2, p2 = torch.empty(T, K, dtype=torch.int32, device="cuda"), torch.empty(T, K, device="cuda")
+    abi.moe_topk(abi.MoeShape.of(T, 1, K, 64, E, 64), z[:T].cuda(), i2, p2)
+    assert torch.equal(i2, idx[:T]) and torch.equal(p2, prob[:T])
+    assert (i2.cpu().numpy() == np.argsort(-z[:T].numpy(), axis=1, kind="stable")[:, :K]).all()
